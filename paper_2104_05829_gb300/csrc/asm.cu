@@ -1245,7 +1245,7 @@ int cheb_w_update(const Level& L, int prec, const void* z, void* x, void* d, dou
 // the seeded start vector in v0, then the largest eigenvalue of the symmetric
 // part of the Hessenberg matrix. FP64 throughout. Synchronous.
 int arnoldi_lmax_asm(Ctx& C, int l, double h1, double h2, const double* v0, int steps, cudaStream_t s,
-                     double* lam) {
+                     double* lam, bool eo) {
   Level& L = C.lev[l];
   const int64_t n = L.nL;
   std::vector<double> H((size_t)(steps + 1) * steps, 0.0);
@@ -1269,7 +1269,7 @@ int arnoldi_lmax_asm(Ctx& C, int l, double h1, double h2, const double* v0, int 
     int k = steps;
     for (int j = 0; j < steps; ++j) {
       const double* vj = V + (size_t)j * n;
-      SEM_TRY(ax_apply(L, SEM_FP64, vj, t, h1, h2, nullptr, s));
+      SEM_TRY(ax_apply(L, SEM_FP64, vj, t, h1, h2, nullptr, s, nullptr, eo));
       SEM_TRY(gs_apply(L, SEM_FP64, t, true, s));
       SEM_TRY(asm_sum(L, SEM_FP64, t, nullptr, w, h1, h2, s));
       SEM_TRY(asm_weight(L, SEM_FP64, w, s));

@@ -293,8 +293,8 @@ int launch_ax_bulk(const Level& L, const float* u, float* w, const GT* G, const 
 
 template <int NP>
 int ax_dispatch_np(const Level& L, int prec, const void* u, void* w, double h1, double h2, const double* h1L,
-                   const double* skip, cudaStream_t s) {
-  if (prec == SEM_FP64) return ax_eo_apply(L, (const double*)u, (double*)w, h1, h2, h1L, skip, s);
+                   const double* skip, cudaStream_t s, bool eo) {
+  if (prec == SEM_FP64) return ax_eo_apply(L, (const double*)u, (double*)w, h1, h2, h1L, skip, s, eo);
   // the bulk copy of u needs a 16-byte aligned source (the per-element sizes are
   // multiples of 16 bytes and the factors are library allocations), so a caller's
   // vector that starts elsewhere, e.g. an offset view, takes the plain-load kernel
@@ -546,14 +546,14 @@ __global__ void k_restrict(int E, const T* __restrict__ bf, const T* __restrict_
   MACRO(2) MACRO(3) MACRO(4) MACRO(5) MACRO(6) MACRO(7) MACRO(8) MACRO(9) MACRO(10) MACRO(11) MACRO(12)
 
 int ax_apply(const Level& L, int prec, const void* u, void* w, double h1, double h2, const double* h1L,
-             cudaStream_t s, const double* skip) {
+             cudaStream_t s, const double* skip, bool eo) {
   if (L.E == 0) return SEM_OK;
   if (prec == SEM_FP32 && !L.G32) { set_detail("FP32 factors were not built"); return SEM_EINVAL; }
   if (prec == SEM_BF16G && !L.G16) { set_detail("BF16 factors were not built"); return SEM_EINVAL; }
   switch (L.NP) {
 #define CASE(NP) \
   case NP:       \
-    return ax_dispatch_np<NP>(L, prec, u, w, h1, h2, h1L, skip, s);
+    return ax_dispatch_np<NP>(L, prec, u, w, h1, h2, h1L, skip, s, eo);
     SEM_NP_CASES(CASE)
 #undef CASE
   }

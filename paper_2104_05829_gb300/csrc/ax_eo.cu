@@ -20,127 +20,11 @@
 //
 // The pair variant keeps every value as an unevaluated sum of two floats
 // (pairs.cuh); the factors are stored pre-split as float2 (hi, lo).
-#include "pairs.cuh"
-#include "sem_internal.cuh"
+#include "eo.cuh"
 
 namespace sem {
 
 namespace {
-
-// ---- arithmetic back ends ------------------------------------------------------
-struct ArF64 {
-  static constexpr bool kPairs = false;
-  using V = double;
-  using GT = double;
-  __device__ static V in(const double* u, size_t i) { return u[i]; }
-  __device__ static void out(double* w, size_t i, V v) { w[i] = v; }
-  __device__ static V gl(const GT* G, size_t i) { return G[i]; }
-  __device__ static V zero() { return 0.0; }
-  __device__ static V add(V a, V b) { return a + b; }
-  __device__ static V sub(V a, V b) { return a - b; }
-  __device__ static V add_u(V a, V b) { return a + b; }
-  __device__ static V sub_u(V a, V b) { return a - b; }
-  __device__ static V mul(V a, V b) { return a * b; }
-  __device__ static V mac(V acc, V a, V b) { return fma(a, b, acc); }
-  __device__ static V tidy(V a) { return a; }
-  __device__ static V tidy_before_add(V a) { return a; }
-  static V host(double x) { return x; }
-};
-
-struct ArPair {
-  static constexpr bool kPairs = true;
-  using V = ff;
-  using GT = float2;
-  __device__ static V in(const double* u, size_t i) { return ff_split(u[i]); }
-  // the FP64 addition in ff_join rounds hi + lo correctly without renormalising first
-  __device__ static void out(double* w, size_t i, V v) { w[i] = ff_join(v); }
-  __device__ static V gl(const GT* G, size_t i) {
-    const float2 g = G[i];
-    return {g.x, g.y};
-  }
-  __device__ static V zero() { return {0.f, 0.f}; }
-  __device__ static V add(V a, V b) { return ff_add(a, b); }
-  __device__ static V sub(V a, V b) { return ff_sub(a, b); }
-  // the additions inside the even-odd line transforms, whose results only enter further
-  // error-free additions and products, skip the renormalisation
-  __device__ static V add_u(V a, V b) { return ff_add_u(a, b); }
-  __device__ static V sub_u(V a, V b) { return ff_sub_u(a, b); }
-  __device__ static V mul(V a, V b) { return ff_mul(a, b); }
-  __device__ static V mac(V acc, V a, V b) { return ff_mac(acc, a, b); }
-  __device__ static V tidy(V a) { return ff_norm(a); }
-  // values that next enter the error-free additions of eo_apply need no renormalising
-  __device__ static V tidy_before_add(V a) { return a; }
-  static V host(double x) { return ff_host_split(x); }
-};
-
-template <class Ar>
-struct EOMat {
-  typename Ar::V ep[36];   // E[a][b], a, b < H
-  typename Ar::V op[36];   // O[a][b]
-  typename Ar::V mc[6];    // D[a][m]: the middle input's weight in ev_a (N even)
-  typename Ar::V mr[6];    // D[m][b]: the middle output's weights on d_b (N even)
-};
-
-template <int NP>
-struct Pad3 {
-  // row stride NP+1 for even NP; plane stride chosen so that rows of
-  // successive planes start on different banks
-  static constexpr int RS = (NP % 2 == 0) ? NP + 1 : NP;
-  static constexpr int PS = NP * RS + ((NP * RS) % 2 == 0 ? 2 : 1);
-  static constexpr int ES = NP * PS;
-};
-
-// Blocks per SM requested from the register allocator: at N = 7 four 192-thread blocks (at
-// most 85 registers; five made the pair kernel spill and run slower). The pair kernel at other
-// orders: three blocks, four at N = 9 (one 100-thread element per block there), against the
-// register allocator's default of one or two blocks of up to 255 registers: at 16.8M points
-// N = 3, 5, 11 took 0.390, 0.416, 1.347 ms with one block and 0.334, 0.371, 0.749 ms with three,
-// and N = 8, 9, 10 took 0.518, 0.848, 0.625 ms with two blocks and 0.453, 0.634 (four),
-// 0.492 ms; the FP64 kernel is bound by its pipe at any occupancy.
-template <class Ar, int NP>
-__host__ __device__ constexpr int eo_min_blocks() {
-  return NP == 8 ? 4 : (Ar::kPairs ? (NP == 10 ? 4 : 3) : 1);
-}
-
-template <int NP>
-__host__ __device__ constexpr int eo_epb() {
-  int e = 256 / (NP * NP);
-  if (e < 1) e = 1;
-  while (e > 1 && (size_t)(3 * e * Pad3<NP>::ES) * 8 > 46 * 1024) --e;
-  return e;
-}
-
-template <class Ar, int NP>
-__device__ __forceinline__ void eo_apply(const EOMat<Ar>& M, const typename Ar::V (&v)[NP],
-                                         typename Ar::V (&o)[NP]) {
-  using V = typename Ar::V;
-  constexpr int H = NP / 2, N = NP - 1;
-  V s[H], d[H];
-#pragma unroll
-  for (int b = 0; b < H; ++b) {
-    s[b] = Ar::add_u(v[b], v[N - b]);
-    d[b] = Ar::sub_u(v[b], v[N - b]);
-  }
-#pragma unroll
-  for (int a = 0; a < H; ++a) {
-    V ev = Ar::mul(M.ep[a * H], s[0]);
-    V od = Ar::mul(M.op[a * H], d[0]);
-#pragma unroll
-    for (int b = 1; b < H; ++b) {
-      ev = Ar::mac(ev, M.ep[a * H + b], s[b]);
-      od = Ar::mac(od, M.op[a * H + b], d[b]);
-    }
-    if (NP % 2 == 1) ev = Ar::mac(ev, M.mc[a], v[H]);
-    o[a] = Ar::add_u(ev, od);
-    o[N - a] = Ar::sub_u(od, ev);
-  }
-  if (NP % 2 == 1) {
-    V m = Ar::mul(M.mr[0], d[0]);
-#pragma unroll
-    for (int b = 1; b < H; ++b) m = Ar::mac(m, M.mr[b], d[b]);
-    o[H] = Ar::tidy(m);
-  }
-}
 
 template <class Ar, int NP, bool VARH1>
 __global__ void __launch_bounds__(NP* NP* eo_epb<NP>(), (eo_min_blocks<Ar, NP>()))
@@ -150,7 +34,7 @@ __global__ void __launch_bounds__(NP* NP* eo_epb<NP>(), (eo_min_blocks<Ar, NP>()
   using V = typename Ar::V;
   constexpr int EPB = eo_epb<NP>();
   constexpr int NP2 = NP * NP, NP3 = NP2 * NP;
-  constexpr int RS = Pad3<NP>::RS, PS = Pad3<NP>::PS, ES = Pad3<NP>::ES;
+  constexpr int ES = Pad3<NP>::ES;
   if (skip && *skip != 0.0) return;
   __shared__ V s_a[EPB * ES];
   __shared__ V s_b[EPB * ES];
@@ -160,115 +44,8 @@ __global__ void __launch_bounds__(NP* NP* eo_epb<NP>(), (eo_min_blocks<Ar, NP>()
   const int ij = tid - le * NP2;
   const int j = ij / NP, i = ij - j * NP;
   const int e = blockIdx.x * EPB + le;
-  const bool active = e < E;
-  V* A = s_a + le * ES;
-  V* B = s_b + le * ES;
-  V* Cc = s_c + le * ES;
-  const size_t ebase = (size_t)e * NP3;
-
-  // phase 0: the element into registers (own t-line) and shared memory
-  V ru[NP];
-#pragma unroll
-  for (int k = 0; k < NP; ++k) {
-    ru[k] = active ? Ar::in(u, ebase + k * NP2 + ij) : Ar::zero();
-    A[k * PS + j * RS + i] = ru[k];
-  }
-  __syncthreads();
-
-  // phase 1: u_t (own line), u_r (row k = i, j), u_s (column k = i, i' = j)
-  V ut[NP];
-  eo_apply<Ar, NP>(Df, ru, ut);
-  {
-    V v[NP], o[NP];
-#pragma unroll
-    for (int l = 0; l < NP; ++l) v[l] = A[i * PS + j * RS + l];
-    eo_apply<Ar, NP>(Df, v, o);
-#pragma unroll
-    for (int l = 0; l < NP; ++l) B[i * PS + j * RS + l] = o[l];
-#pragma unroll
-    for (int l = 0; l < NP; ++l) v[l] = A[i * PS + l * RS + j];
-    eo_apply<Ar, NP>(Df, v, o);
-#pragma unroll
-    for (int l = 0; l < NP; ++l) Cc[i * PS + l * RS + j] = o[l];
-  }
-  __syncthreads();
-
-  // phase 2: pointwise G-combine, in place
-  if (active) {
-    const typename Ar::GT* Ge = G + (size_t)e * 7 * NP3 + ij;
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      const int o = k * NP2;
-      const V ur = B[k * PS + j * RS + i], us = Cc[k * PS + j * RS + i], uq = ut[k];
-      const V g11 = Ar::gl(Ge, 0 * NP3 + o), g12 = Ar::gl(Ge, 1 * NP3 + o), g13 = Ar::gl(Ge, 2 * NP3 + o);
-      const V g22 = Ar::gl(Ge, 3 * NP3 + o), g23 = Ar::gl(Ge, 4 * NP3 + o), g33 = Ar::gl(Ge, 5 * NP3 + o);
-      V wr = Ar::mac(Ar::mac(Ar::mul(g11, ur), g12, us), g13, uq);
-      V ws = Ar::mac(Ar::mac(Ar::mul(g12, ur), g22, us), g23, uq);
-      V wt = Ar::mac(Ar::mac(Ar::mul(g13, ur), g23, us), g33, uq);
-      if (VARH1) {
-        const V hh = Ar::in(h1L, ebase + o + ij);
-        wr = Ar::mul(wr, hh);
-        ws = Ar::mul(ws, hh);
-        wt = Ar::mul(wt, hh);
-      }
-      B[k * PS + j * RS + i] = Ar::tidy_before_add(wr);
-      Cc[k * PS + j * RS + i] = Ar::tidy_before_add(ws);
-      ut[k] = Ar::tidy_before_add(wt);
-    }
-  }
-  __syncthreads();
-
-  // phase 3a: D_t^T on the own line, D_r^T on row (k = i, j) -> A
-  V ot[NP];
-  eo_apply<Ar, NP>(Dt, ut, ot);
-  {
-    V v[NP], o[NP];
-#pragma unroll
-    for (int l = 0; l < NP; ++l) v[l] = B[i * PS + j * RS + l];
-    eo_apply<Ar, NP>(Dt, v, o);
-#pragma unroll
-    for (int l = 0; l < NP; ++l) A[i * PS + j * RS + l] = o[l];
-  }
-  __syncthreads();
-  // phase 3b: D_s^T on column (k = i, i' = j) -> B
-  {
-    V v[NP], o[NP];
-#pragma unroll
-    for (int l = 0; l < NP; ++l) v[l] = Cc[i * PS + l * RS + j];
-    eo_apply<Ar, NP>(Dt, v, o);
-#pragma unroll
-    for (int l = 0; l < NP; ++l) B[i * PS + l * RS + j] = o[l];
-  }
-  __syncthreads();
-
-  // phase 4: w = h1 (D^T G D u) + h2 B u
-  if (active) {
-    const typename Ar::GT* Be = G + (size_t)e * 7 * NP3 + 6 * NP3 + ij;
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      const V st = Ar::add_u(Ar::add_u(A[k * PS + j * RS + i], B[k * PS + j * RS + i]), ot[k]);
-      const V hb = Ar::mul(Ar::mul(h2, Ar::gl(Be, k * NP2)), ru[k]);
-      Ar::out(w, ebase + k * NP2 + ij, VARH1 ? Ar::add(st, hb) : Ar::mac(hb, h1, st));
-    }
-  }
-}
-
-template <class Ar>
-void make_eo(const double* D, int NP, bool transpose, EOMat<Ar>& M) {
-  const int H = NP / 2, N = NP - 1, m = NP / 2;
-  auto at = [&](int a, int b) { return transpose ? D[b * NP + a] : D[a * NP + b]; };
-  for (int q = 0; q < 36; ++q) M.ep[q] = M.op[q] = Ar::host(0.0);
-  for (int q = 0; q < 6; ++q) M.mc[q] = M.mr[q] = Ar::host(0.0);
-  for (int a = 0; a < H; ++a)
-    for (int b = 0; b < H; ++b) {
-      M.ep[a * H + b] = Ar::host(0.5 * (at(a, b) + at(a, N - b)));
-      M.op[a * H + b] = Ar::host(0.5 * (at(a, b) - at(a, N - b)));
-    }
-  if (NP % 2 == 1)
-    for (int a = 0; a < H; ++a) {
-      M.mc[a] = Ar::host(at(a, m));
-      M.mr[a] = Ar::host(at(m, a));
-    }
+  eo_element<Ar, NP, VARH1>(true, e < E, i, j, (size_t)e * NP3, u, w, G + (size_t)e * 7 * NP3, Df, Dt, h1, h2, h1L,
+                            s_a + le * ES, s_b + le * ES, s_c + le * ES);
 }
 
 template <class Ar>
@@ -306,20 +83,23 @@ __global__ void k_split_pairs(int64_t n, const double* __restrict__ G, float2* _
 
 }  // namespace
 
-// FP64 element operator (even-odd contractions).
+// FP64 element operator: in digits where the level has fixed-point factors (ax_dig.cu), else, or with eo, by even-odd
+// contractions.
 int ax_eo_apply(const Level& L, const double* u, double* w, double h1, double h2, const double* h1L,
-                const double* skip, cudaStream_t s) {
+                const double* skip, cudaStream_t s, bool eo) {
+  if (L.Gx && !eo) return ax_dig_apply(L, 0, L.E, u, w, h1, h2, h1L, skip, s);
   return eo_launch<ArF64>(L, u, w, L.G, h1, h2, h1L, skip, s);
 }
 
 // FP64-accurate element operator in FP32-pair arithmetic (scalar h1, or a nodal h1L, split
-// into pairs as it is read).
+// into pairs as it is read); in digits where those are faster, unless eo.
 int ax_pairs_apply(const Level& L, const double* u, double* w, double h1, double h2, const double* h1L,
-                   cudaStream_t s) {
-  if (!L.G2) {
+                   cudaStream_t s, bool eo) {
+  if (!L.pairs) {
     set_detail("FP32-pair factors were not built");
     return SEM_EINVAL;
   }
+  if (dig_for_pairs(L) && !eo) return ax_dig_apply(L, 0, L.E, u, w, h1, h2, h1L, nullptr, s);
   return eo_launch<ArPair>(L, u, w, L.G2, h1, h2, h1L, nullptr, s);
 }
 
@@ -328,22 +108,23 @@ int ax_pairs_apply(const Level& L, const double* u, double* w, double h1, double
 int ax_eo_apply_range(const Level& L, int e0, int e1, const double* u, double* w, double h1, double h2,
                       const double* h1L, bool pairs, cudaStream_t s) {
   if (e1 <= e0) return SEM_OK;
+  if (pairs && !L.pairs) {
+    set_detail("FP32-pair factors not built");
+    return SEM_EINVAL;
+  }
+  if (pairs ? dig_for_pairs(L) : L.Gx != nullptr) return ax_dig_apply(L, e0, e1 - e0, u, w, h1, h2, h1L, nullptr, s);
   const size_t off = (size_t)e0 * L.NP * L.NP * L.NP;
   Level V = L;
   V.E = e1 - e0;
   V.nL = (int64_t)V.E * L.NP * L.NP * L.NP;
-  if (pairs) {
-    if (!L.G2) {
-      set_detail("FP32-pair factors not built");
-      return SEM_EINVAL;
-    }
+  if (pairs)
     return eo_launch<ArPair>(V, u + off, w + off, L.G2 + 7 * off, h1, h2, h1L ? h1L + off : nullptr, nullptr, s);
-  }
   return eo_launch<ArF64>(V, u + off, w + off, L.G + 7 * off, h1, h2, h1L ? h1L + off : nullptr, nullptr, s);
 }
 
 // (hi, lo) FP32 split of the FP64 factors for the pair kernel.
 int pairs_build(Level& L, cudaStream_t s) {
+  L.pairs = true;
   if (!L.G2) {
     cudaError_t e = cudaMalloc((void**)&L.G2, 7 * L.nL * sizeof(float2) + 16);
     if (e != cudaSuccess) {

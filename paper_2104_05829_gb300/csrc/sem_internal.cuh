@@ -14,6 +14,8 @@
 
 namespace sem {
 
+struct DigTab;   // dig.cuh
+
 // ----------------------------------------------------------------------------
 // Error plumbing: every entry point returns a status; the last failure's text
 // is kept per host thread for sem_last_error_detail.
@@ -77,6 +79,12 @@ struct Level {
   float* G32 = nullptr;
   __nv_bfloat16* G16 = nullptr;
   float2* G2 = nullptr;        // (hi, lo) FP32 split of G for the pair-arithmetic kernel
+  bool pairs = false;          // SEM_BUILD_PAIRS was asked for: SEM_AX_PAIRS / SEM_FP64P calls are accepted
+  // fixed-point factors of the digit kernel (ax_dig.cu; null: the even-odd kernels run)
+  int2* Gx = nullptr;          // [E][6][NP][NP][NP rounded up to even] (signed low word, high word)
+  int32_t* gexp = nullptr;     // [E] exponents
+  DigTab* dig = nullptr;
+  int dig_kexp = 0;
   // coordinates, ids and Dirichlet flags as given (fine) or derived (coarse)
   double *x = nullptr, *y = nullptr, *z = nullptr;
   int64_t* gid = nullptr;
@@ -220,8 +228,9 @@ constexpr int RED_BLOCKS = 1216;
 constexpr int RED_THREADS = 256;
 
 // ---- ax.cu
+// eo: the FP64 operator in its even-odd FP64 (or FP32-pair) form, not in digits
 int ax_apply(const Level& L, int prec, const void* u, void* w, double h1, double h2, const double* h1L,
-             cudaStream_t s, const double* skip = nullptr);
+             cudaStream_t s, const double* skip = nullptr, bool eo = false);
 // a nodal field of level F at the GLL points of the next coarser level C (setup.cu), the way
 // the coarse coordinates are formed (the fine element interpolant at the coarse points)
 int interp_nodal(const Level& F, const Level& C, const double* f, double* c, cudaStream_t s);
@@ -231,16 +240,24 @@ int geom_compute(Level& L, int* d_bad, cudaStream_t s);
 
 // ---- ax_eo.cu (FP64 element operator, even-odd contractions)
 int ax_eo_apply(const Level& L, const double* u, double* w, double h1, double h2, const double* h1L,
-                const double* skip, cudaStream_t s);
+                const double* skip, cudaStream_t s, bool eo = false);
 
 // elements [e0, e1) of the level only (u, w, h1L: whole-level L-vectors)
 int ax_eo_apply_range(const Level& L, int e0, int e1, const double* u, double* w, double h1, double h2,
                       const double* h1L, bool pairs, cudaStream_t s);
 
+// ---- ax_dig.cu (FP64 element operator in integer digits on the tensor cores)
+int dig_build(Level& L, cudaStream_t s);
+// N = 7: the digit kernel answers the FP32-pair calls too, with more bits and in less time (32^3: 306 against 366 us); at
+// other orders its lines are padded to eight points and the pair kernel is the faster one (N = 5, 43^3: 617 against 350 us).
+inline bool dig_for_pairs(const Level& L) { return L.Gx && L.NP == 8; }
+int ax_dig_apply(const Level& L, int e0, int E, const double* u, double* w, double h1, double h2, const double* h1L,
+                 const double* skip, cudaStream_t s);
+
 // ---- ax_eo.cu (FP32-pair variant)
 int pairs_build(Level& L, cudaStream_t s);
 int ax_pairs_apply(const Level& L, const double* u, double* w, double h1, double h2, const double* h1L,
-                   cudaStream_t s);
+                   cudaStream_t s, bool eo = false);
 
 // ---- coarse_pipe.cu: recursive coordinate bisection (host): el[0..n) goes to parts
 // part0 .. part0 + parts - 1 (el_off[part] = first position), sizes within one of each
@@ -299,7 +316,7 @@ int asm_weight(const Level& L, int prec, void* z, cudaStream_t s);
 int cheb_w_update(const Level& L, int prec, const void* z, void* x, void* d, double c1, double c2, bool first,
                   bool x_zero, cudaStream_t s);
 int arnoldi_lmax_asm(Ctx& C, int l, double h1, double h2, const double* v0, int steps, cudaStream_t s,
-                     double* lam);
+                     double* lam, bool eo);
 
 // ---- advect.cu: dealiased advection operator
 int advect_build(Ctx& C, cudaStream_t s);

@@ -140,9 +140,9 @@ double tridiag_max_eig(const std::vector<double>& a, const std::vector<double>& 
 
 // the preconditioner's operator on level l (a nodal h1 of the preconditioner replaces h1)
 int level_op(Ctx& C, int l, int prec, const void* x, void* w, double h1, double h2, cudaStream_t s,
-             const double* skip = nullptr) {
+             const double* skip = nullptr, bool eo = false) {
   const Level& L = C.lev[l];
-  SEM_TRY(ax_apply(L, prec, x, w, h1, h2, C.pc_nodal ? L.h1n : nullptr, s, skip));
+  SEM_TRY(ax_apply(L, prec, x, w, h1, h2, C.pc_nodal ? L.h1n : nullptr, s, skip, eo));
   return gs_apply_skip(L, prec, w, true, skip, s);
 }
 
@@ -161,7 +161,7 @@ int level_dinv(Ctx& C, int l, double h1, double h2, const double* h1L, double* o
   return dinv_finalize(L, out, out32, s);
 }
 
-int lanczos(Ctx& C, int l, double h1, double h2, cudaStream_t s, double* lam) {
+int lanczos(Ctx& C, int l, double h1, double h2, cudaStream_t s, double* lam, bool eo) {
   Level& L = C.lev[l];
   const int64_t n = L.nL;
   double *v = L.vb, *vprev = L.vx, *w = L.vw, *t = L.vd;
@@ -177,7 +177,7 @@ int lanczos(Ctx& C, int l, double h1, double h2, cudaStream_t s, double* lam) {
   for (int j = 0; j < C.opts.lanczos_steps; ++j) {
     k_sqrt_mul<<<vgrid(n), 256, 0, s>>>(n, L.dinv, v, t);
     SEM_LAUNCH_CHECK();
-    SEM_TRY(level_op(C, l, SEM_FP64, t, w, h1, h2, s));
+    SEM_TRY(level_op(C, l, SEM_FP64, t, w, h1, h2, s, nullptr, eo));
     k_lanczos_w<<<vgrid(n), 256, 0, s>>>(n, L.dinv, w, vprev, beta);
     SEM_LAUNCH_CHECK();
     SEM_TRY(dot_owner(C, L, SEM_FP64, w, v, d_tmp, s));
@@ -345,6 +345,7 @@ int precond_setup(Ctx& C, double h1, double h2, int prec, cudaStream_t s, const 
   // level operators take it point by point (the scalar h1 becomes 1)
   C.pc_nodal = h1L != nullptr;
   C.pc_h1L = h1L;
+  const bool eo = !h1L && prec != SEM_FP64;   // the eigenvalue bounds of an FP32 V-cycle keep their last bit (see solve_impl)
   if (h1L) {
     h1 = 1.0;
     for (int l = 0; l < C.nlevels; ++l) {
@@ -378,9 +379,9 @@ int precond_setup(Ctx& C, double h1, double h2, int prec, cudaStream_t s, const 
       SEM_TRY(schwarz_build(C, L, s));
       k_lanczos_start<<<vgrid(L.nL), 256, 0, s>>>(L.nL, L.label, L.dmask, C.opts.lanczos_seed, L.vb);
       SEM_LAUNCH_CHECK();
-      SEM_TRY(arnoldi_lmax_asm(C, l, h1, h2, L.vb, C.opts.lanczos_steps, s, &L.lmax));
+      SEM_TRY(arnoldi_lmax_asm(C, l, h1, h2, L.vb, C.opts.lanczos_steps, s, &L.lmax, eo));
     } else {
-      SEM_TRY(lanczos(C, l, h1, h2, s, &L.lmax));
+      SEM_TRY(lanczos(C, l, h1, h2, s, &L.lmax, eo));
     }
   }
   SEM_CUDA_TRY(cudaStreamSynchronize(s));
@@ -473,7 +474,7 @@ int check_level(Ctx* C, int level) {
 int check_prec(Ctx* C, int level, int prec) {
   const Level& L = C->lev[level];
   if (prec == SEM_FP64) return SEM_OK;
-  if (prec == SEM_FP64P && L.G2) return SEM_OK;
+  if (prec == SEM_FP64P && L.pairs) return SEM_OK;
   if (prec == SEM_FP32 && L.G32) return SEM_OK;
   if (prec == SEM_BF16G && L.G16) return SEM_OK;
   set_detail("precision %d not available (not built or unknown)", prec);
@@ -743,14 +744,19 @@ int solve_impl(Ctx* C, Proj* P, const double* f, const sem_coef* c, double tol, 
     return SEM_EINVAL;
   }
   const bool pairs = (rhs_flags & SEM_OUTER_PAIRS) != 0;
-  if (pairs && !C->lev[0].G2) {
+  if (pairs && !C->lev[0].pairs) {
     set_detail("sem_solve: SEM_OUTER_PAIRS needs the pair factors (SEM_BUILD_PAIRS)");
     return SEM_EINVAL;
   }
-  // outer operator R QQ^T A_L p (FP64 or FP32-pair element kernel)
+  // Outer operator R QQ^T A_L p. An FP32 V-cycle turns a last-bit change of its input into other FP32 roundings and another
+  // number of coarse iterations, and the solution then changes by a part of the solve's own error (3e-8 to 9e-8 at
+  // tol = 1e-8, 24^3, whichever two FP64-accurate operators are compared). So such a solve to a loose tolerance keeps the
+  // even-odd operator and its earlier result; below 1e-9 (5e-12 apart at 1e-10), with an FP64 V-cycle and with Jacobi the digit
+  // operator runs.
+  const bool eo = precond == SEM_PC_PMG && prec != SEM_FP64 && tol > 1e-9;
   auto outer_ax = [&](const double* in, double* out, const double* skip, cudaStream_t st) -> int {
-    if (pairs) SEM_TRY(ax_pairs_apply(C->lev[0], in, out, c->h1, c->h2, c->h1_L, st));
-    else SEM_TRY(ax_apply(C->lev[0], SEM_FP64, in, out, c->h1, c->h2, c->h1_L, st, skip));
+    if (pairs) SEM_TRY(ax_pairs_apply(C->lev[0], in, out, c->h1, c->h2, c->h1_L, st, eo));
+    else SEM_TRY(ax_apply(C->lev[0], SEM_FP64, in, out, c->h1, c->h2, c->h1_L, st, skip, eo));
     return gs_apply_skip(C->lev[0], SEM_FP64, out, true, skip, st);
   };
   Level& L = C->lev[0];
