@@ -155,7 +155,8 @@ __global__ void __launch_bounds__(DigShape<NP>::T, dig_min_blocks<NP>())
     um = max(um, s_max[0][t]);
     if (VARH1) hm = max(hm, s_max[1][t]);
   }
-  const int eu = um ? (int)(um >> 20) : 1023;               // biased exponent of the largest |u|
+  // biased exponent of the largest |u|, one more where its fixed-point form would reach 2^63 (1 - 2^-7)
+  const int eu = um ? (int)((um + 0x4000) >> 20) : 1023;
   const int eh = VARH1 ? (hm ? (int)(hm >> 20) - 1022 : 0) : 0;   // |h1| < 2^eh
   // exponent of the result's unit before the shift by the derivatives' size (at most 32)
   const int ex = ge + eh + eu - 1023 - kexp - DIG_SH2 - 12;
@@ -348,7 +349,7 @@ __global__ void __launch_bounds__(128)
   if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = m;
   ok = __syncthreads_and(ok);
   m = fmax(fmax(s_m[0], s_m[1]), fmax(s_m[2], s_m[3]));
-  const int ge = ok && m > 0.0 ? ilogb(m) + 1 : DIG_BAD;
+  const int ge = ok && m > 0.0 ? ilogb(m * (1.0 + 0x1p-5)) + 1 : DIG_BAD;   // the fluxes stay below 2^63 (1 - 2^-7)
   const bool take = ge != DIG_BAD && abs(ge) < 400;
   if (threadIdx.x == 0) gexp[e] = take ? ge : DIG_BAD;
   const double sc = take ? ldexp(1.0, 62 - ge) : 0.0;
@@ -458,7 +459,7 @@ int dig_build_np(Level& L, cudaStream_t s) {
   for (int st = 0; st < 2; ++st)
     for (int a = 0; a < NP; ++a)
       for (int d = 0; d < 8; ++d)
-        for (int b = 0; b < NP; ++b) z[st][a][d] += 128 * H.dg[st][a][b][d];
+        for (int b = 0; b < NP; ++b) z[st][a][d] += H.dg[st][a][b][d];
   for (int a = 0; a < 8; ++a) {
     T.a[a] = a < NP ? H.a[a] : 0;
     T.nk0[a] = 0ull - dig_merge_zero(z[0][a], DIG_SH1);

@@ -10,10 +10,10 @@
 // 64), which leaves an error of about 2^-60 of the element's largest term, against 2^-53 of every
 // partial sum in FP64.
 //
-// * Digits of a value. The byte b of the sign-flipped number is put into an FP16 register half
-//   as it is: as a subnormal its value is b 2^-24, so one byte permute gives two digits, with no
-//   conversion. The flipped sign adds 2^63 to every value; what that adds to an output is a constant
-//   of the matrix row, which dig_merge's nk takes out again.
+// * Digits of a value. 128 is added to every byte (one 64-bit addition), and a byte b = digit + 128 is put into an FP16
+//   register half as it is: as a subnormal its value is b 2^-24, so one byte permute gives two digits, with no
+//   conversion. What the 128s add to an output is a constant of the matrix row, which dig_merge's nk takes out again
+//   (exactly: an all-zero line gives zero).
 // * Two digits of a value lie beside each other along the mma's depth (16 = 8 points x 2 digits),
 //   the two matrix digits that belong with them likewise, and the sixteen rows are the eight outputs
 //   twice, with the matrix digits shifted by one: rows 0-7 give the odd weights 2q+1, rows 8-15 the even
@@ -48,10 +48,11 @@ __device__ __forceinline__ void dig_mma(float (&d)[4], const uint32_t a0, const 
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
 }
 
-// A fixed-point value is kept with its sign flipped (dig_flip); dig_pair(x, n) is its digits 2n+1 (low half) and 2n
-// (high half) in FP16.
+// A fixed-point value is kept with 128 added to each of its bytes (dig_flip; |x| < 2^63 (1 - 2^-7) keeps that in 64 bits): its
+// digits, byte - 128, lie in -128..127 around zero, so that the digit products that are dropped have no mean. dig_pair(x, n) is
+// the bytes 2n+1 (low half) and 2n (high half) in FP16.
 __device__ __forceinline__ unsigned long long dig_flip(const long long x) {
-  return (unsigned long long)x ^ 0x8000000000000000ull;
+  return (unsigned long long)x + 0x8080808080808080ull;
 }
 __device__ __forceinline__ uint32_t dig_pair(const unsigned long long x, const int n) {
   return __byte_perm(n < 2 ? (uint32_t)(x >> 32) : (uint32_t)x, 0, n & 1 ? 0x4140 : 0x4342);
@@ -208,6 +209,30 @@ __device__ __forceinline__ void dig_lines_both(unsigned long long (&v)[4], const
   for (int r = 0; r < 4; ++r) v[r] = dig_merge<SH>(s[r], dig_two_both(t[1], f[1], r), dig_two_both(t[0], f[0], r), r & 1 ? nk.y : nk.x);
 }
 
+// One group of eight lines as columns, all weights at once: f[q] = weights 2q+1 ([0], [1]) and 2q ([2], [3]) of output g for
+// lines 2c and 2c+1; b[x]: the digits of point 2c+x of line g. START: the sums begin at 0.75, else they go on.
+template <bool START>
+__device__ __forceinline__ void dig_sums(float (&f)[4][4], const uint4 (&D)[4], const DigPack (&b)[2],
+                                         const DigStart& z) {
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+#pragma unroll
+    for (int q = 3; q >= m; --q) {
+      const int n = q - m;
+      float(&o)[4] = f[q];
+      if (START && m == 0)
+        dig_mma(o, D[0].x, D[0].y, D[0].z, D[0].w, b[0].p[n], b[1].p[n], z.z[0], z.z[1], z.z[2], z.z[3]);
+      else
+        dig_mma(o, D[m].x, D[m].y, D[m].z, D[m].w, b[0].p[n], b[1].p[n], o[0], o[1], o[2], o[3]);
+    }
+}
+template <int SH>
+__device__ __forceinline__ unsigned long long dig_merge4(const float (&f)[4][4], const int x,
+                                                         const unsigned long long nk) {
+  const DigAcc a = {dig_two(f[0][2 + x], f[0][x]), dig_two(f[3][2 + x], f[3][x])};
+  return dig_merge<SH>(a, dig_two(f[1][2 + x], f[1][x]), dig_two(f[2][2 + x], f[2][x]), nk);
+}
+
 // |x| as a fixed-point number of 63 bits with binary exponent `top` (the biased exponent of the
 // element's largest value) at bit 62, the sign applied; the bits below are dropped.
 __device__ __forceinline__ long long dig_fix(const double x, const int top) {
@@ -240,8 +265,10 @@ inline uint16_t half_of(int v) {
   return (uint16_t)((v < 0 ? 0x8000 : 0) | ((ex + 15) << 10) | ((a << 10 >> ex) & 0x3ff));
 }
 
-// What a merge gives, without nk, where every value is zero (digits 128, 0, ...): s[d] = 128 x the sum of the row's digits d.
-inline unsigned long long dig_merge_zero(const int64_t (&s)[8], int SH) {
+// What a merge gives, without nk, where every value is zero (bytes 128): r[d] = the sum of the row's matrix digits d.
+inline unsigned long long dig_merge_zero(const int64_t (&r0)[8], int SH) {
+  int64_t s[8], c = 0;
+  for (int d = 0; d < 8; ++d) s[d] = 128 * (c += r0[d]);
   auto two = [&](int q) { return (uint32_t)(((0x3f400000 + s[2 * q]) << 8) + 0x3f400000 + s[2 * q + 1]); };
   const unsigned long long r = (((unsigned long long)two(0) << 32) | two(2)) + ((unsigned long long)two(1) << 16);
   return (r << (SH - 40)) + (two(3) >> (56 - SH));

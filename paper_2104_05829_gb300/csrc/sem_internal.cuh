@@ -14,7 +14,8 @@
 
 namespace sem {
 
-struct DigTab;   // dig.cuh
+struct DigTab;      // dig.cuh
+struct AdvDigTab;   // advect_dig.cu
 
 // ----------------------------------------------------------------------------
 // Error plumbing: every entry point returns a status; the last failure's text
@@ -179,6 +180,13 @@ struct AdvData {
   float2 *Im2 = nullptr, *Dq2 = nullptr;
   double hIm[14 * 9] = {0};   // host copies (nq <= 14, N + 1 <= 9)
   double hDq[14 * 14] = {0};
+  double hwq[14] = {0};
+  // fixed-point factors and tables of the digit kernel (advect_dig.cu; built on the first FP64 or pair evaluation)
+  bool dig_tried = false;
+  int2* Gqx = nullptr;        // [E][9][nq][lines (a, b)] (signed low word, high word)
+  int32_t* gqexp = nullptr;   // [E]
+  AdvDigTab* dig = nullptr;
+  int dig_ebase = 0;
   // characteristics substeps: inverse assembled mass and RK workspace (allocated on first use)
   double* minv = nullptr;     // [nL] 1 / (QQ^T B_L)
   float* minv32 = nullptr;
@@ -324,6 +332,11 @@ void advect_free(AdvData& A);
 int advect_apply(Ctx& C, int prec, const void* c, const void* u, void* w, int ncomp, cudaStream_t s);
 int char_advance(Ctx& C, int prec, const void* c0, const void* c1, void* w, int ncomp, double t0, double t1,
                  int nsub, cudaStream_t s);
+
+// ---- advect_dig.cu: the same in integer digits (FP64 data)
+int advect_dig_build(AdvData& A, const Level& L, cudaStream_t s);
+int advect_dig_apply(const Level& L, const AdvData& A, const double* c, const double* u, double* w, int ncomp,
+                     cudaStream_t s);
 
 // ---- proj.cu: projection of successive right-hand sides
 struct Proj;
