@@ -3,7 +3,7 @@
 // Dot products are unique-node inner products of continuous L-vectors: the sum
 // over one owner copy of every non-Dirichlet node (equal to the counting-
 // weighted sum of the paper's w-weighted reductions, but with one product per
-// node). Reductions are deterministic: a fixed grid of RED_BLOCKS blocks walks
+// node). Reductions are deterministic: a grid fixed by the vector's length walks
 // the vector with a fixed stride, each block reduces in a fixed shuffle tree,
 // and the last block to finish (atomic ticket) adds the block partials in
 // index order and finalises the Krylov scalars on the device. Nothing spins.
@@ -361,10 +361,10 @@ int vec_copy_convert(const void* src, int sprec, void* dst, int dprec, int64_t n
 
 int dot_owner(Ctx& C, const Level& L, int prec, const void* a, const void* b, double* d_out, cudaStream_t s) {
   if (prec == SEM_FP64)
-    k_dot<double><<<RED_BLOCKS, RED_THREADS, 0, s>>>(L.nL, (const double*)a, (const double*)b, L.owner,
+    k_dot<double><<<red_grid(L.nL), RED_THREADS, 0, s>>>(L.nL, (const double*)a, (const double*)b, L.owner,
                                                      C.red_part, C.red_ticket, d_out);
   else
-    k_dot<float><<<RED_BLOCKS, RED_THREADS, 0, s>>>(L.nL, (const float*)a, (const float*)b, L.owner, C.red_part,
+    k_dot<float><<<red_grid(L.nL), RED_THREADS, 0, s>>>(L.nL, (const float*)a, (const float*)b, L.owner, C.red_part,
                                                     C.red_ticket, d_out);
   SEM_LAUNCH_CHECK();
   return SEM_OK;
@@ -394,11 +394,11 @@ int mul_counting_weight(const Level& L, int prec, const void* in, void* out, cud
 int pcg_begin_tol(Ctx& C, const Level& L, int prec, const void* b, const void* w, void* x, void* r,
                   const void* dinv, void* p, double* sc, double tol, cudaStream_t s, const double* bbref) {
   if (prec == SEM_FP64)
-    k_pcg_begin<double><<<RED_BLOCKS, RED_THREADS, 0, s>>>(L.nL, (const double*)b, (const double*)w, (double*)x,
+    k_pcg_begin<double><<<red_grid(L.nL), RED_THREADS, 0, s>>>(L.nL, (const double*)b, (const double*)w, (double*)x,
                                                            (double*)r, (const double*)dinv, (double*)p, L.owner,
                                                            C.red_part, C.red_ticket, sc, tol, bbref);
   else
-    k_pcg_begin<float><<<RED_BLOCKS, RED_THREADS, 0, s>>>(L.nL, (const float*)b, (const float*)w, (float*)x,
+    k_pcg_begin<float><<<red_grid(L.nL), RED_THREADS, 0, s>>>(L.nL, (const float*)b, (const float*)w, (float*)x,
                                                           (float*)r, (const float*)dinv, (float*)p, L.owner,
                                                           C.red_part, C.red_ticket, sc, tol, bbref);
   SEM_LAUNCH_CHECK();
@@ -407,10 +407,10 @@ int pcg_begin_tol(Ctx& C, const Level& L, int prec, const void* b, const void* w
 
 int kr_alpha(Ctx& C, const Level& L, int prec, const void* p, const void* w, double* sc, cudaStream_t s) {
   if (prec == SEM_FP64)
-    k_alpha<double><<<RED_BLOCKS, RED_THREADS, 0, s>>>(L.nL, (const double*)p, (const double*)w, L.owner,
+    k_alpha<double><<<red_grid(L.nL), RED_THREADS, 0, s>>>(L.nL, (const double*)p, (const double*)w, L.owner,
                                                        C.red_part, C.red_ticket, sc);
   else
-    k_alpha<float><<<RED_BLOCKS, RED_THREADS, 0, s>>>(L.nL, (const float*)p, (const float*)w, L.owner, C.red_part,
+    k_alpha<float><<<red_grid(L.nL), RED_THREADS, 0, s>>>(L.nL, (const float*)p, (const float*)w, L.owner, C.red_part,
                                                       C.red_ticket, sc);
   SEM_LAUNCH_CHECK();
   return SEM_OK;
@@ -419,11 +419,11 @@ int kr_alpha(Ctx& C, const Level& L, int prec, const void* p, const void* w, dou
 int kr_update_jacobi(Ctx& C, const Level& L, int prec, void* x, const void* p, void* r, const void* w,
                      const void* dinv, double* sc, cudaStream_t s) {
   if (prec == SEM_FP64)
-    k_update_jacobi<double><<<RED_BLOCKS, RED_THREADS, 0, s>>>(L.nL, (double*)x, (const double*)p, (double*)r,
+    k_update_jacobi<double><<<red_grid(L.nL), RED_THREADS, 0, s>>>(L.nL, (double*)x, (const double*)p, (double*)r,
                                                                (const double*)w, (const double*)dinv, L.owner,
                                                                C.red_part, C.red_ticket, sc);
   else
-    k_update_jacobi<float><<<RED_BLOCKS, RED_THREADS, 0, s>>>(L.nL, (float*)x, (const float*)p, (float*)r,
+    k_update_jacobi<float><<<red_grid(L.nL), RED_THREADS, 0, s>>>(L.nL, (float*)x, (const float*)p, (float*)r,
                                                               (const float*)w, (const float*)dinv, L.owner,
                                                               C.red_part, C.red_ticket, sc);
   SEM_LAUNCH_CHECK();
@@ -445,10 +445,10 @@ int kr_direction_jacobi(const Level& L, int prec, void* p, const void* r, const 
 int kr_update_flex(Ctx& C, const Level& L, double* x, const double* p, double* r, const double* w, void* rb,
                    int rb_prec, double* sc, cudaStream_t s) {
   if (rb_prec == SEM_FP64)
-    k_update_flex<double><<<RED_BLOCKS, RED_THREADS, 0, s>>>(L.nL, x, p, r, w, (double*)rb, L.owner, C.red_part,
+    k_update_flex<double><<<red_grid(L.nL), RED_THREADS, 0, s>>>(L.nL, x, p, r, w, (double*)rb, L.owner, C.red_part,
                                                              C.red_ticket, sc);
   else
-    k_update_flex<float><<<RED_BLOCKS, RED_THREADS, 0, s>>>(L.nL, x, p, r, w, (float*)rb, L.owner, C.red_part,
+    k_update_flex<float><<<red_grid(L.nL), RED_THREADS, 0, s>>>(L.nL, x, p, r, w, (float*)rb, L.owner, C.red_part,
                                                             C.red_ticket, sc);
   SEM_LAUNCH_CHECK();
   return SEM_OK;
@@ -457,10 +457,10 @@ int kr_update_flex(Ctx& C, const Level& L, double* x, const double* p, double* r
 int kr_beta_flex(Ctx& C, const Level& L, const void* z, int z_prec, const double* r, const double* w, double* sc,
                  cudaStream_t s) {
   if (z_prec == SEM_FP64)
-    k_beta_flex<double><<<RED_BLOCKS, RED_THREADS, 0, s>>>(L.nL, (const double*)z, r, w, L.owner, C.red_part,
+    k_beta_flex<double><<<red_grid(L.nL), RED_THREADS, 0, s>>>(L.nL, (const double*)z, r, w, L.owner, C.red_part,
                                                            C.red_ticket, sc);
   else
-    k_beta_flex<float><<<RED_BLOCKS, RED_THREADS, 0, s>>>(L.nL, (const float*)z, r, w, L.owner, C.red_part,
+    k_beta_flex<float><<<red_grid(L.nL), RED_THREADS, 0, s>>>(L.nL, (const float*)z, r, w, L.owner, C.red_part,
                                                           C.red_ticket, sc);
   SEM_LAUNCH_CHECK();
   return SEM_OK;

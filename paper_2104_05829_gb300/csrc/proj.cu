@@ -100,7 +100,7 @@ __global__ void k_proj_add(int64_t n, double* __restrict__ u, const double* __re
 template <int NV>
 void launch_dots(int64_t n, const double* X, int64_t ld, const double* y, const double* ea, const double* eb,
                  const uint8_t* own, double* part, unsigned* ticket, double* c, double* extra, cudaStream_t s) {
-  k_proj_dots<NV><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, X, ld, y, ea, eb, own, part, ticket, c, extra);
+  k_proj_dots<NV><<<red_grid(n), RED_THREADS, 0, s>>>(n, X, ld, y, ea, eb, own, part, ticket, c, extra);
 }
 
 template <int NV>
@@ -108,13 +108,13 @@ void launch_combine(int dot, int64_t n, const double* X, const double* AX, int64
                     const double* xb, double* xo, const double* rb, double* ro, const uint8_t* own, double* part,
                     unsigned* ticket, double* nrm, cudaStream_t s) {
   if (dot == 0)
-    k_proj_combine<NV, 0><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, X, AX, ld, c, sx, xb, xo, rb, ro, own, part, ticket,
+    k_proj_combine<NV, 0><<<red_grid(n), RED_THREADS, 0, s>>>(n, X, AX, ld, c, sx, xb, xo, rb, ro, own, part, ticket,
                                                             nrm);
   else if (dot == 1)
-    k_proj_combine<NV, 1><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, X, AX, ld, c, sx, xb, xo, rb, ro, own, part, ticket,
+    k_proj_combine<NV, 1><<<red_grid(n), RED_THREADS, 0, s>>>(n, X, AX, ld, c, sx, xb, xo, rb, ro, own, part, ticket,
                                                             nrm);
   else
-    k_proj_combine<NV, 2><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, X, AX, ld, c, sx, xb, xo, rb, ro, own, part, ticket,
+    k_proj_combine<NV, 2><<<red_grid(n), RED_THREADS, 0, s>>>(n, X, AX, ld, c, sx, xb, xo, rb, ro, own, part, ticket,
                                                             nrm);
 }
 
