@@ -791,6 +791,8 @@ int solve_impl(Ctx* C, Proj* P, const double* f, const sem_coef* c, double tol, 
     SEM_TRY(level_dinv(*C, 0, c->h1, c->h2, c->h1_L, dinv, nullptr, s));
     SEM_TRY(pcg_begin_tol(*C, L, SEM_FP64, b, x0 ? w : nullptr, u, C->r, dinv, C->p, sc, tol, s, bbref));
     const int batch = 8;
+    // the one-launch form (b is read no more: its array holds the points' copies), at most 1,024 iterations a launch
+    bool one = pairs ? dig_for_pairs(L) : L.Gx != nullptr;
     int launched = 0;
     while (true) {
       SEM_TRY(read_scalars(*C, 0, s));
@@ -806,6 +808,15 @@ int solve_impl(Ctx* C, Proj* P, const double* f, const sem_coef* c, double tol, 
       if (launched >= maxit) {
         rc = SEM_ENOTCONV;
         break;
+      }
+      if (one) {
+        const int nb = std::min(1024, maxit - launched);
+        SEM_TRY(jacobi_dig_solve(*C, L, u, C->r, C->p, w, dinv, c->h1, c->h2, c->h1_L, reinterpret_cast<int2*>(C->t), sc,
+                                 nb, launched == 0, s, &one));
+        if (one) {
+          launched += nb;
+          continue;
+        }
       }
       const int nb = std::min(batch, maxit - launched);
       for (int q = 0; q < nb; ++q) {
