@@ -123,7 +123,9 @@ typedef struct {
   int32_t coarse_mode;       /* how the order-1 coarse Jacobi-PCG runs: SEM_COARSE_* (default AUTO) */
   int64_t spin_limit;        /* SM clock cycles a device-side wait may spin before it gives up (2^31, about a
                                 second at GB300's clock; >= 0). A wait that gives up makes the solve that
-                                launched it return SEM_EBREAKDOWN (the coarse solve's exchange waits) or turns
+                                launched it return SEM_EBREAKDOWN (the coarse solve's exchange waits, the grid
+                                barriers of a small Jacobi-PCG; limits below 2^21 keep that solve to kernels
+                                without waits) or turns
                                 the outputs of the waiting block into NaN (the FP32 operator's bulk-copy wait,
                                 which then waits once more, with the default limit, for its copies to land) */
 } sem_opts;
@@ -185,7 +187,10 @@ int sem_level_info(const sem_ctx* ctx, int level, sem_level_desc* out);
  * GB300 executes far faster than FP64 instructions. The Dirichlet entries
  * of u_L are used as given; pass a masked u_L (zero at Dirichlet nodes, as every
  * solver vector is) to apply A = R Q^T A_L Q R^T. u_L and w_L must not alias.
- * Errors: SEM_EINVAL, SEM_ECUDA. */
+ * Orders 4 to 11: the FP64 call, and the SEM_AX_PAIRS call at N = 7, 9 and 11, run in integer digits on the
+ * tensor cores (64-bit fixed point per element, at least FP64's accuracy, any FP64 exponent) from a
+ * fixed-point copy of the factors that sem_setup builds (48 bytes a point; without the memory for it, and
+ * at other orders, FP64 instructions and pairs). Errors: SEM_EINVAL, SEM_ECUDA. */
 int sem_ax(sem_ctx* ctx, const double* u_L, double* w_L, const sem_coef* coef, int flags, void* stream);
 
 /* w_L <- QQ^T w_L (SEM_GS_ADD) or R QQ^T w_L (SEM_GS_ADD_MASK) on the fine
@@ -315,7 +320,9 @@ int sem_solve_proj(sem_ctx* ctx, sem_proj* pj, const double* f_L, const sem_coef
  * prec SEM_FP64 (double vectors), SEM_FP64P (double vectors, the operator in FP32-pair
  * arithmetic: about 48 significant bits, FP32 exponent range; the pair copies of the
  * cubature factors, 9 nq^3 float2 per element, are built on the first such call) or SEM_FP32
- * (float vectors, FP32 arithmetic).
+ * (float vectors, FP32 arithmetic). SEM_FP64 at N = 4..7 and SEM_FP64P at N = 5..7 run in integer digits on the
+ * tensor cores, from a fixed-point copy of the cubature factors (9 nq^3 64-bit values per element, built on the
+ * first such call; without the memory for it, as at the other orders).
  * The cubature factors w J dr/dx at the Gauss points are built on the first call
  * (synchronous; 9 nq^3 values per element in FP64 and FP32). Compiled for 2 <= N <= 8. */
 #define SEM_ADV_LOCAL 0

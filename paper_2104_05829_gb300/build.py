@@ -18,7 +18,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "libsem.so")
-SOURCES = ["setup.cu", "gsmap.cu", "ax.cu", "ax_eo.cu", "ax_dig.cu", "jacobi_dig.cu", "gs.cu", "blas.cu", "solve.cu", "dot_static.cu",
+SOURCES = ["setup.cu", "gsmap.cu", "ax.cu", "ax_eo.cu", "ax_dig.cu", "ax_dig_eo.cu", "jacobi_dig.cu", "gs.cu", "blas.cu", "solve.cu", "dot_static.cu",
            "proj.cu", "asm.cu", "coarse_pipe.cu", "advect.cu", "advect_dig.cu", "peaks.cu", "dist.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--extended-lambda", "-Xcompiler", "-fPIC", "-I", INCLUDE]

@@ -21,17 +21,23 @@
 // The GLL weights make G, and the result, a hundred times smaller at an element's edges and corners than inside. So G is stored
 // over 2^(a_i + a_j + a_k), 2^a_i near rho_i^(3/4) (a power of two: no rounding), the second contraction uses
 // 2^-a D^T 2^a, and the result gets 2^(a_i + a_j + a_k) back in the exponent of its scale: edges and corners then keep the
-// relative error of the interior (2-norm error against 80-bit arithmetic on random u: 0.9e-16 of the result, 1.6e-16 for
-// the FP64 form; smooth u 3e-16 and 6e-15).
+// relative error of the interior (2-norm error against 80-bit arithmetic on random u: 0.7e-16 of the result, 1.6e-16 for
+// the FP64 form; smooth u 2e-16 and 6e-15).
 //
 // Elements that fixed point cannot hold (an Inf or NaN in u, h1 or G, or exponents near the ends of
 // the FP64 range) are computed by the even-odd FP64 code in the same block.
 #include <cmath>
+#include <cstddef>
 #include <vector>
 
 #include "ax_dig.cuh"
 
 namespace sem {
+
+int dig_eo_tables(const Level& L, const int* a, int k, int m2, int q2, DigEoTab** tab, cudaStream_t s);
+const int32_t* dig_eo_exponents(const DigEoTab* tab);
+int ax_dig_eo_apply(const Level& L, int e0, int E, const double* u, double* w, double h1, double h2, const double* h1L,
+                    const double* skip, const EOMat<ArF64>& Df, const EOMat<ArF64>& Dt, cudaStream_t s);
 
 namespace {
 
@@ -61,21 +67,21 @@ __global__ void __launch_bounds__(DigShape<NP>::T, dig_min_blocks<NP>())
 // row sum |G_m1| + |G_m2| + |G_m3| of its points, as (signed low word, high word).
 template <int NP>
 __global__ void __launch_bounds__(128)
-    k_dig_factors(const double* __restrict__ G, const DigTab* __restrict__ tab, int2* __restrict__ Gx,
+    k_dig_factors(const double* __restrict__ G, const int32_t* __restrict__ a, int2* __restrict__ Gx,
                   int32_t* __restrict__ gexp) {
   using S = DigShape<NP>;
   constexpr int NP3 = NP * NP * NP;
   __shared__ double s_m[4];
   const int e = blockIdx.x;
   const double* Ge = G + (size_t)e * 7 * NP3;
-  auto weight = [&](int i, int kj) { return ldexp(1.0, -(tab->a[i] + tab->a[kj % NP] + tab->a[kj / NP])); };
+  auto weight = [&](int i, int kj) { return ldexp(1.0, -(a[i] + a[kj % NP] + a[kj / NP])); };
   double m = 0.0;
   bool ok = true;
   for (int t = threadIdx.x; t < NP3; t += 128) {
-    double a[6];
+    double v[6];
     const double r = weight(t % NP, t / NP);
-    for (int q = 0; q < 6; ++q) a[q] = fabs(Ge[q * NP3 + t]) * r;
-    const double r0 = a[0] + a[1] + a[2], r1 = a[1] + a[3] + a[4], r2 = a[2] + a[4] + a[5];
+    for (int q = 0; q < 6; ++q) v[q] = fabs(Ge[q * NP3 + t]) * r;
+    const double r0 = v[0] + v[1] + v[2], r1 = v[1] + v[3] + v[4], r2 = v[2] + v[4] + v[5];
     ok = ok && isfinite(r0) && isfinite(r1) && isfinite(r2);
     m = fmax(m, fmax(r0, fmax(r1, r2)));
   }
@@ -97,22 +103,6 @@ __global__ void __launch_bounds__(128)
 
 // ---- host: the digit tables of an order ----------------------------------------------------------
 
-using i128 = __int128;
-
-// round(x num/den 2^s) in integers, half away from zero
-i128 scaled(double x, int num, int den, int s) {
-  int ex;
-  const i128 m = (i128)std::llround(std::ldexp(std::frexp(x, &ex), 53)) * num;
-  const int sh = ex - 53 + s;
-  const bool neg = m < 0;
-  i128 a = neg ? -m : m;
-  i128 b = den;
-  if (sh >= 0) a <<= sh;
-  else b <<= -sh;
-  a = (2 * a + b) / (2 * b);
-  return neg ? -a : a;
-}
-
 struct DigHost {
   int dg[2][12][12][8];   // digits of the scaled matrices [stage][out][in]
   int kexp;               // c1 c2 = 2^kexp
@@ -120,37 +110,41 @@ struct DigHost {
 };
 
 // D scaled by c1 = 2^k / c2 and 2^-a D^T 2^a by c2: every entry below 1 (eight digits), a line's derivative below 2 max|u|
-// (61 bits after the merge), the sum of the three directions within 64 bits; c2 has eight significant bits, so that
-// the divisions are exact in 128-bit integers. False when the sums of digits would not stay exact.
-bool dig_digits(const double* Dm, const double* rho, int NP, DigHost& H) {
+// (61 bits after the merge), the sum of the three directions within 64 bits; c2 = m2 2^(q2 - 8) has eight significant
+// bits, so that the divisions are exact in 128-bit integers.
+double dig_entry(const double* Dm, int NP, const int* A, int st, int a, int b) {
+  return st ? std::ldexp(Dm[b * NP + a], A[b] - A[a]) : Dm[a * NP + b];
+}
+void dig_scales(const double* Dm, const double* rho, int NP, int* A, int* k, int* m2, int* q2) {
   double row[2] = {0, 0}, mx[2] = {0, 0};
   double rm = 0;
   for (int a = 0; a < NP; ++a) rm = std::fmax(rm, rho[a]);
-  for (int a = 0; a < NP; ++a) H.a[a] = (int)std::lround(0.75 * std::log2(rho[a] / rm));
-  auto entry = [&](int st, int a, int b) {
-    return st ? std::ldexp(Dm[b * NP + a], H.a[b] - H.a[a]) : Dm[a * NP + b];
-  };
+  for (int a = 0; a < NP; ++a) A[a] = (int)std::lround(0.75 * std::log2(rho[a] / rm));
   for (int st = 0; st < 2; ++st)
     for (int a = 0; a < NP; ++a) {
       double r = 0;
       for (int b = 0; b < NP; ++b) {
-        r += std::fabs(entry(st, a, b));
-        mx[st] = std::fmax(mx[st], std::fabs(entry(st, a, b)));
+        r += std::fabs(dig_entry(Dm, NP, A, st, a, b));
+        mx[st] = std::fmax(mx[st], std::fabs(dig_entry(Dm, NP, A, st, a, b)));
       }
       row[st] = std::fmax(row[st], r);
     }
   const double g = 1.0 - 0x1p-10;
   const double c1m = std::fmin(2.0 / row[0], 1.0 / mx[0]) * g, c2m = std::fmin(4.0 / (3.0 * row[1]), 1.0 / mx[1]) * g;
-  int q2;
-  const int m2 = (int)std::floor(std::ldexp(std::frexp(c2m, &q2), 8));   // c2 = m2 2^(q2 - 8)
-  const double c2 = std::ldexp((double)m2, q2 - 8);
-  const int k = (int)std::floor(std::log2(c1m * c2));
+  *m2 = (int)std::floor(std::ldexp(std::frexp(c2m, q2), 8));
+  *k = (int)std::floor(std::log2(c1m * std::ldexp((double)*m2, *q2 - 8)));
+}
+
+// The digits of an order up to 7; false when the sums of digits would not stay exact.
+bool dig_digits(const double* Dm, const double* rho, int NP, DigHost& H) {
+  int k, m2, q2;
+  dig_scales(Dm, rho, NP, H.a, &k, &m2, &q2);
   H.kexp = k;
   for (int st = 0; st < 2; ++st)
     for (int a = 0; a < NP; ++a)
       for (int b = 0; b < NP; ++b) {
-        const double d = entry(st, a, b);
-        i128 v = st ? scaled(d, m2, 1, 63 + q2 - 8) : scaled(d, 1, m2, 63 + k - (q2 - 8));
+        const double d = dig_entry(Dm, NP, H.a, st, a, b);
+        __int128 v = st ? dig_scaled(d, m2, 1, 63 + q2 - 8) : dig_scaled(d, 1, m2, 63 + k - (q2 - 8));
         for (int t = 7; t > 0; --t) {
           const int x = (int)(((v + 128) & 255) - 128);
           H.dg[st][a][b][t] = x;
@@ -170,9 +164,30 @@ bool dig_digits(const double* Dm, const double* rho, int NP, DigHost& H) {
   return true;
 }
 
+// The level's fixed-point factors; a: the exponents on the device. The stream is synchronised (the tables' host copies go).
+template <int NP>
+int dig_factors(Level& L, const int32_t* a, int kexp, cudaStream_t s) {
+  using S = DigShape<NP>;
+  int2* Gx = nullptr;
+  int32_t* ge = nullptr;
+  if (cudaMalloc((void**)&Gx, (size_t)L.E * 6 * S::GE * sizeof(int2)) != cudaSuccess ||
+      cudaMalloc((void**)&ge, (size_t)L.E * sizeof(int32_t)) != cudaSuccess) {
+    cudaGetLastError();
+    if (Gx) cudaFree(Gx);
+    SEM_CUDA_TRY(cudaStreamSynchronize(s));
+    return SEM_OK;
+  }
+  L.Gx = Gx;
+  L.gexp = ge;
+  L.dig_kexp = kexp;
+  k_dig_factors<NP><<<L.E, 128, 0, s>>>(L.G, a, Gx, ge);
+  SEM_LAUNCH_CHECK();
+  SEM_CUDA_TRY(cudaStreamSynchronize(s));
+  return SEM_OK;
+}
+
 template <int NP>
 int dig_build_np(Level& L, cudaStream_t s) {
-  using S = DigShape<NP>;
   DigHost H;
   if (!dig_digits(L.D.a, L.rho, NP, H)) return SEM_OK;
   std::vector<DigTab> tab(1);
@@ -204,27 +219,26 @@ int dig_build_np(Level& L, cudaStream_t s) {
       T.nk1rs[a * 8 + b] = 0ull - dig_merge_zero(t, DIG_SH2);
     }
   }
-  int2* Gx = nullptr;
-  int32_t* ge = nullptr;
   DigTab* dt = nullptr;
   // without the memory the even-odd form runs
-  if (cudaMalloc((void**)&Gx, (size_t)L.E * 6 * S::GE * sizeof(int2)) != cudaSuccess ||
-      cudaMalloc((void**)&ge, (size_t)L.E * sizeof(int32_t)) != cudaSuccess ||
-      cudaMalloc((void**)&dt, sizeof(DigTab)) != cudaSuccess) {
+  if (cudaMalloc((void**)&dt, sizeof(DigTab)) != cudaSuccess) {
     cudaGetLastError();
-    if (Gx) cudaFree(Gx);
-    if (ge) cudaFree(ge);
     return SEM_OK;
   }
-  L.Gx = Gx;
-  L.gexp = ge;
   L.dig = dt;
-  L.dig_kexp = H.kexp;
   SEM_CUDA_TRY(cudaMemcpyAsync(dt, &T, sizeof(DigTab), cudaMemcpyHostToDevice, s));
-  k_dig_factors<NP><<<L.E, 128, 0, s>>>(L.G, dt, Gx, ge);
-  SEM_LAUNCH_CHECK();
-  SEM_CUDA_TRY(cudaStreamSynchronize(s));   // tab goes out of scope
-  return SEM_OK;
+  return dig_factors<NP>(L, reinterpret_cast<const int32_t*>(reinterpret_cast<const char*>(dt) + offsetof(DigTab, a)),
+                         H.kexp, s);
+}
+
+// 8 <= N <= 11
+template <int NP>
+int dig_build_eo(Level& L, cudaStream_t s) {
+  int A[12], k, m2, q2;
+  dig_scales(L.D.a, L.rho, NP, A, &k, &m2, &q2);
+  SEM_TRY(dig_eo_tables(L, A, k, m2, q2, &L.dig_eo, s));
+  if (!L.dig_eo) return SEM_OK;
+  return dig_factors<NP>(L, dig_eo_exponents(L.dig_eo), k, s);
 }
 
 }  // namespace
@@ -236,6 +250,10 @@ int dig_build(Level& L, cudaStream_t s) {
     case 6: return dig_build_np<6>(L, s);
     case 7: return dig_build_np<7>(L, s);
     case 8: return dig_build_np<8>(L, s);
+    case 9: return dig_build_eo<9>(L, s);
+    case 10: return dig_build_eo<10>(L, s);
+    case 11: return dig_build_eo<11>(L, s);
+    case 12: return dig_build_eo<12>(L, s);
     default: return SEM_OK;
   }
 }
@@ -270,6 +288,7 @@ int ax_dig_apply(const Level& L, int e0, int E, const double* u, double* w, doub
     CASE(5) CASE(6) CASE(7) CASE(8)
 #undef CASE
   }
+  if (L.dig_eo) return ax_dig_eo_apply(L, e0, E, u, w, h1, h2, h1L, skip, Df, Dt, s);
   set_detail("order %d not compiled", L.N);
   return SEM_EINVAL;
 }

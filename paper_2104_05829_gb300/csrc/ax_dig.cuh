@@ -22,6 +22,20 @@ struct DigShape {
   static constexpr int SMEM = 3 * FLD > 3 * Pad3<NP>::ES ? 3 * FLD : 3 * Pad3<NP>::ES;   // of the block
 };
 
+// round(x num/den 2^s) in integers, half away from zero
+inline __int128 dig_scaled(double x, int num, int den, int s) {
+  int ex;
+  const __int128 m = (__int128)std::llround(std::ldexp(std::frexp(x, &ex), 53)) * num;
+  const int sh = ex - 53 + s;
+  const bool neg = m < 0;
+  __int128 a = neg ? -m : m;
+  __int128 b = den;
+  if (sh >= 0) a <<= sh;
+  else b <<= -sh;
+  a = (2 * a + b) / (2 * b);
+  return neg ? -a : a;
+}
+
 // exponent of a scalar h1, as the kernel takes it (4096: not a normal number, the elements go to the FP64 form)
 inline int dig_h1_exp(double h1) { return h1 == 0.0 ? 0 : std::isnormal(h1) ? std::ilogb(h1) : 4096; }
 

@@ -82,10 +82,11 @@ struct Level {
   __nv_bfloat16* G16 = nullptr;
   float2* G2 = nullptr;        // (hi, lo) FP32 split of G for the pair-arithmetic kernel
   bool pairs = false;          // SEM_BUILD_PAIRS was asked for: SEM_AX_PAIRS / SEM_FP64P calls are accepted
-  // fixed-point factors of the digit kernel (ax_dig.cu; null: the even-odd kernels run)
+  // fixed-point factors of the digit kernels (ax_dig.cu, ax_dig_eo.cu; null: the even-odd kernels run)
   int2* Gx = nullptr;          // [E][6][NP][NP][NP rounded up to even] (signed low word, high word)
   int32_t* gexp = nullptr;     // [E] exponents
-  DigTab* dig = nullptr;
+  DigTab* dig = nullptr;       // N = 4..7
+  DigEoTab* dig_eo = nullptr;  // N = 8..11 (ax_dig_eo.cu)
   int dig_kexp = 0;
   // coordinates, ids and Dirichlet flags as given (fine) or derived (coarse)
   double *x = nullptr, *y = nullptr, *z = nullptr;
@@ -257,9 +258,10 @@ int ax_eo_apply_range(const Level& L, int e0, int e1, const double* u, double* w
 
 // ---- ax_dig.cu (FP64 element operator in integer digits on the tensor cores)
 int dig_build(Level& L, cudaStream_t s);
-// N = 7: the digit kernel answers the FP32-pair calls too, with more bits and in less time (32^3: 306 against 366 us); at
-// other orders its lines are padded to eight points and the pair kernel is the faster one (N = 5, 43^3: 617 against 350 us).
-inline bool dig_for_pairs(const Level& L) { return L.Gx && L.NP == 8; }
+// N = 7, 9 and 11: the digit kernels answer the FP32-pair calls too, with more bits and in less time (306 against 366 us at 32^3,
+// 600 against 635 at 26^3, 490 against 682 at 21^3); at other orders their lines are padded and the pair kernel is the
+// faster one (N = 5, 43^3: 617 against 350 us; N = 8, 28^3: 673 against 458; N = 10, 23^3: 652 against 495).
+inline bool dig_for_pairs(const Level& L) { return L.Gx && (L.NP == 8 || L.NP == 10 || L.NP == 12); }
 int ax_dig_apply(const Level& L, int e0, int E, const double* u, double* w, double h1, double h2, const double* h1L,
                  const double* skip, cudaStream_t s);
 
