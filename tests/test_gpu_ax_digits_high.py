@@ -28,7 +28,7 @@ def test_orders_and_coefficients(N, nodal):
         ref = O.ax_local(u.reshape(B.shape), G, B, lev.D, np.reshape(h1, B.shape) if nodal else h1, h2)
         for pairs in (False, True):
             w = H(ctx.ax(T(u), h1=1.0 if nodal else h1, h1_L=T(h1) if nodal else None, h2=h2, assemble=False, pairs=pairs))
-            assert relmax(w, ref.ravel()) < (TOL if not pairs or N % 2 else 5e-12)
+            assert relmax(w, ref.ravel()) < (TOL if not pairs or N == 11 else 5e-12)
     ctx.close()
 
 
@@ -49,4 +49,12 @@ def test_scale_zero_and_elements_of_the_fp64_form(N):
     v[3] = np.inf
     bad = H(ctx.ax(T(v), h2=0.5, assemble=False)).reshape(4, -1)
     assert not np.all(np.isfinite(bad[0])) and np.array_equal(bad[1:], w.reshape(4, -1)[1:])
+    ctx.close()
+
+
+def test_pair_calls_take_the_digits_of_a_large_mesh():
+    mesh = si.box_mesh((13, 13, 13), 9, warp=0.1, perm_seed=0)
+    ctx = ctx_for(mesh, prec_copies=4)
+    u = T(si.uniform_field(mesh, 2, continuous=False))
+    assert np.array_equal(H(ctx.ax(u, h2=0.5, assemble=False)), H(ctx.ax(u, h2=0.5, assemble=False, pairs=True)))
     ctx.close()
