@@ -917,7 +917,7 @@ def main():
     if e2e is not None:
         line["e2e"] = e2e
     if not args.no_variants:
-        # the other element kernel on the same inputs (reported, not the headline)
+        # the other call on the same inputs (reported, not the headline; at N = 7 one kernel answers both)
         other = not pairs
         fn = lambda: ctx.ax(u, w, h1=1.0, h2=0.5, assemble=True, pairs=other)
         for _ in range(3):
