@@ -327,7 +327,7 @@ int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, do
   a.idx = L.seg_idx;
   a.part = C.red_part;
   a.sc = sc;
-  unsigned* sync = reinterpret_cast<unsigned*>(C.scal + 2 * S_NSLOTS);   // a spare slot set
+  unsigned* sync = reinterpret_cast<unsigned*>(C.scal + 4 * S_NSLOTS);   // its own slot set
   a.bar = sync;
   a.err = reinterpret_cast<int*>(sync + 1);
   a.spin = L.spin_limit;
@@ -348,7 +348,12 @@ int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, do
   }
   SEM_CUDA_TRY(cudaMemsetAsync(sync, 0, 2 * sizeof(unsigned), s));
   void* args[] = {&a, &Df, &Dt};
-  SEM_CUDA_TRY(cudaLaunchCooperativeKernel(f, dim3(L.E), dim3(threads), args, 0, s));
+  const cudaError_t rc = cudaLaunchCooperativeKernel(f, dim3(L.E), dim3(threads), args, 0, s);
+  if (rc == cudaErrorCooperativeLaunchTooLarge) {   // a part of the device only (MPS, green contexts): the launches
+    cudaGetLastError();
+    return SEM_OK;
+  }
+  SEM_CUDA_TRY(rc);
   *used = true;
   return SEM_OK;
 }

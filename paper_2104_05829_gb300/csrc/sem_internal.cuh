@@ -204,7 +204,7 @@ struct Ctx {
   // deterministic reduction scratch
   double* red_part = nullptr;       // [RED_BLOCKS * 4]
   unsigned int* red_ticket = nullptr;
-  double* scal = nullptr;           // [4 * S_NSLOTS]: outer, coarse, spare
+  double* scal = nullptr;           // [5 * S_NSLOTS]: outer, coarse, sem_dot, Lanczos, one-launch Jacobi-PCG
   double* h_scal = nullptr;         // pinned mirror
   // fine-level FP64 solver workspace
   double *r = nullptr, *z = nullptr, *p = nullptr, *w = nullptr, *t = nullptr;

@@ -506,8 +506,8 @@ int sem_setup(const sem_mesh* m, const sem_opts* opts_in, sem_ctx** out) {
   STEP(dmalloc(&C->red_ticket, 1));
   STEP(dmalloc(&C->cg_err, 1));
   CUSTEP(cudaMemsetAsync(C->red_ticket, 0, sizeof(unsigned), s));
-  STEP(dmalloc(&C->scal, 4 * S_NSLOTS));
-  CUSTEP(cudaMemsetAsync(C->scal, 0, 4 * S_NSLOTS * sizeof(double), s));
+  STEP(dmalloc(&C->scal, 5 * S_NSLOTS));
+  CUSTEP(cudaMemsetAsync(C->scal, 0, 5 * S_NSLOTS * sizeof(double), s));
   CUSTEP(cudaMallocHost((void**)&C->h_scal, 4 * S_NSLOTS * sizeof(double)));
   STEP(dmalloc(&C->r, nL));
   STEP(dmalloc(&C->z, nL));
