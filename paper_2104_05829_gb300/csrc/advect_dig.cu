@@ -168,7 +168,9 @@ __global__ void __launch_bounds__(DigAdv<NP>::T, 2)
     par ^= 1;
     return m;
   };
-  // a field as sign-flipped fixed point, its largest value's exponent at bit 62 - down
+  // a field as sign-flipped fixed point, its largest value's exponent at bit 62 - down: |u| < 2^62, |c| < 2^61. A pass's row sums
+  // are below 2 and its unit is doubled, so every later operand of dig_flip keeps that bound; conv, at most 1.16 2^61 (the row
+  // sums of I, I, DI over the three directions, N = 6), is below 2^62 once shifted.
   auto load = [&](const double* v, int ex, int down) {
     for (int q = threadIdx.x; q < NP3; q += S::T) {
       const int k = q / NP2, j = q / NP % NP, i = q % NP;

@@ -152,7 +152,7 @@ __device__ __forceinline__ bool dig_element(const int e, const double* __restric
     return false;
   }
 
-  // digits of u; derivatives along r from the lane's own digits
+  // digits of u (below 2^63 (1 - 2^-7): eu); derivatives along r from the lane's own digits
   const DigStart zs;
   unsigned long long Vr[4], Vs[4], Vt[4];   // derivatives at point 2c + x of plane p: [2p + x], two's complement
   {
@@ -247,6 +247,7 @@ __device__ __forceinline__ bool dig_element(const int e, const double* __restric
             mad_wide_s(ah[2], gl(q2),
                        mad_wide_s(al[1], gh(q1),
                                   mad_wide_s(ah[1], gl(q1), mad_wide_s(al[0], gh(q0), mul_wide_s(ah[0], gl(q0)))))));
+        // a derivative (times h1) below 2^61, factors below 2^62 / (1 + 2^-5) in sum (k_dig_factors): below 2^63 / (1 + 2^-5)
         return dig_flip((hh << 4) + (m >> 28));
       };
       fr[p][x] = flux(0, 1, 2);

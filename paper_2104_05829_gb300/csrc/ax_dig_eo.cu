@@ -3,9 +3,9 @@
 // What bounds it: the FP64 form (ax_eo.cu) issues an FP64 instruction every 16 cycles: 2,368 us at 26^3, N = 9, against 187 us
 // for its bytes. Here it is instruction issue and the mma.sync chains (ncu, 16^3, N = 9: issue 56 %, tensor pipe 30 %, 755 warp
 // instructions for 32 points; 917 with one loop over all groups and 8-byte stores). Element kernel, about 16 million points, FP64 form ->
-// this: N = 8 1841 -> 673 us, N = 9 2368 -> 600, N = 10 1872 -> 652, N = 11 2460 -> 490. (The FP32-pair kernel: 458, 634, 495, 682.)
-// Error against 128-bit arithmetic, 2-norm, random u: 0.5e-16 to 0.75e-16 (FP64 form 1.4e-16 to 1.65e-16); smooth u 1.0e-15 to 3.8e-15
-// (6.8e-15 to 1.2e-14).
+// this: N = 8 1841 -> 675 us, N = 9 2368 -> 602, N = 10 1872 -> 653, N = 11 2460 -> 491. (The FP32-pair kernel: 458, 634, 495, 682.)
+// Error against 128-bit arithmetic, 2-norm, 4x3x4 warped elements: random u 0.57e-16 to 0.7e-16 (FP64 form 1.4e-16 to 1.65e-16); linear,
+// quadratic and smooth u 0.54e-15 (N = 8) to 5.3e-15 (N = 11) (FP64 form 2.9e-15 to 1.8e-14).
 //
 // A line of NP = 9..12 points is two contractions of at most six: the sums v[b] + v[N-b] with the even part of the matrix, the
 // differences with the odd part. Each fits an mma's eight points and eight outputs, where the lines as they are would take
@@ -55,6 +55,9 @@ constexpr int dig_eo_min_blocks() {
 }
 
 // The lines of direction DIR (0: i, 1: j, 2: k), group by group: src and dst may be the same field. g0: this warp's first group.
+// Bounds: u comes below 2^62 (1 - 2^-7) (half of what the exponent eu leaves), a flux shifted by sh below 2^62 / (1 + 2^-6), so the
+// sums s and d that dig_flip takes are below 2^63 (1 - 2^-7) and 2^63 / (1 + 2^-6). ev and od together stay below 2^60 (derivatives)
+// and 2^62 / 3 (each direction of the result) by the scales of the matrices.
 template <int NP, int SH, int DIR>
 __device__ __forceinline__ uint32_t dig_eo_lines(const unsigned long long* src, unsigned long long* dst, const int g0,
                                                  const uint4 (&De)[4], const uint4 (&Do)[4], const unsigned long long nke,
@@ -267,14 +270,18 @@ __global__ void __launch_bounds__(DigEoShape<NP>::T, dig_eo_min_blocks<NP>())
     F[i] = f0;
     F[S::FLD + i] = f1;
     F[2 * S::FLD + i] = f2;
-    fm |= dig_size(f0) | dig_size(f1) | dig_size(f2);
+    fm = max(max(fm, dig_size(f0)), max(dig_size(f1), dig_size(f2)));
   }
-  fm = __reduce_or_sync(0xffffffffu, fm);
+  fm = __reduce_max_sync(0xffffffffu, fm);
   if (lane == 0) s_max[0][wp] = fm;
   __syncthreads();
 #pragma unroll
-  for (int t = 0; t < S::NW; ++t) fm |= s_max[0][t];
-  const int sf = max(__clz(fm) - 2, 0);   // the largest flux below 2^62 (1 - 2^-7): to 2^61
+  for (int t = 0; t < S::NW; ++t) fm = max(fm, s_max[0][t]);
+  // |flux| < (fm + 1) 2^32, and fm + fm / 64 + 1 below 2^(30 - sf) makes (fm + 1) (1 + 2^-6) at most 2^(30 - sf): shifted by sf, a
+  // flux stays below 2^62 / (1 + 2^-6), and the sum or difference of two mirror points (dig_eo_lines), 0.9847 2^63 at most, within
+  // dig_flip's bound. Mirror fluxes are equal wherever u is linear, so that the sums do come this close. Unshifted (sf = 0) a flux
+  // is below 2^62 / (1 + 2^-5) by the exponent of the factors.
+  const int sf = max(__clz(fm + (fm >> 6) + 1) - 2, 0);
   dig_eo_pass<NP, 1>(U, F, tab, sf, zs);
   __syncthreads();
 

@@ -48,8 +48,8 @@ __device__ __forceinline__ void dig_mma(float (&d)[4], const uint32_t a0, const 
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
 }
 
-// A fixed-point value is kept with 128 added to each of its bytes (dig_flip; |x| < 2^63 (1 - 2^-7) keeps that in 64 bits): its
-// digits, byte - 128, lie in -128..127 around zero, so that the digit products that are dropped have no mean. dig_pair(x, n) is
+// A fixed-point value is kept with 128 added to each of its bytes (dig_flip; x < 2^63 (1 - 2^-8) keeps that in 64 bits, and every
+// use says what bounds its operand): its digits, byte - 128, lie in -128..127 around zero, so that the digit products that are dropped have no mean. dig_pair(x, n) is
 // the bytes 2n+1 (low half) and 2n (high half) in FP16.
 __device__ __forceinline__ unsigned long long dig_flip(const long long x) {
   return (unsigned long long)x + 0x8080808080808080ull;
