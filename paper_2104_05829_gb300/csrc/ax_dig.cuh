@@ -36,6 +36,18 @@ inline __int128 dig_scaled(double x, int num, int den, int s) {
   return neg ? -a : a;
 }
 
+// A nodal h1 is kept in 61 bits below the element's largest, so its values keep FP64's 53 bits down to 2^-8 of that; an element whose
+// h1 spans more (a jump of a material, say) is computed in FP64, which keeps every value's own bits. dig_h1_low is largest for the
+// smallest |h1| that is not zero (a zero is exact in both); dig_h1_wide takes the block's largest high word of |h1| and dig_h1_low.
+constexpr int DIG_H1_SPAN = 61 - 53;
+__device__ __forceinline__ uint32_t dig_h1_low(const double h1) {
+  const uint32_t a = (uint32_t)__double2hiint(h1) & 0x7fffffffu;
+  return (a | (uint32_t)__double2loint(h1)) ? 0x7fffffffu - a : 0u;
+}
+__device__ __forceinline__ bool dig_h1_wide(const uint32_t high, const uint32_t low) {
+  return (int)(high >> 20) - (int)((0x7fffffffu - low) >> 20) > DIG_H1_SPAN;
+}
+
 // exponent of a scalar h1, as the kernel takes it (4096: not a normal number, the elements go to the FP64 form)
 inline int dig_h1_exp(double h1) { return h1 == 0.0 ? 0 : std::isnormal(h1) ? std::ilogb(h1) : 4096; }
 
@@ -116,19 +128,28 @@ __device__ __forceinline__ bool dig_element(const int e, const double* __restric
     if (VARH1) ld2(h1L, p, hv[p]);
   }
   const int ge = gexp[e];
-  uint32_t um = 0, hm = 0;
+  uint32_t um = 0, hm = 0, hl = 0;
 #pragma unroll
   for (int p = 0; p < 2; ++p)
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
       um = max(um, (uint32_t)__double2hiint(uv[p][x]) & 0x7fffffffu);
-      if (VARH1) hm = max(hm, (uint32_t)__double2hiint(hv[p][x]) & 0x7fffffffu);
+      if (VARH1) {
+        hm = max(hm, (uint32_t)__double2hiint(hv[p][x]) & 0x7fffffffu);
+        hl = max(hl, dig_h1_low(hv[p][x]));
+      }
     }
   um = __reduce_max_sync(0xffffffffu, um);
-  if (VARH1) hm = __reduce_max_sync(0xffffffffu, hm);
+  if (VARH1) {
+    hm = __reduce_max_sync(0xffffffffu, hm);
+    hl = __reduce_max_sync(0xffffffffu, hl);
+  }
   if (lane == 0) {
     s_max[0][wp] = um;
-    if (VARH1) s_max[1][wp] = hm;
+    if (VARH1) {
+      s_max[1][wp] = hm;
+      s_max[3][wp] = hl;
+    }
   }
   uint4 D[4];
 #pragma unroll
@@ -137,7 +158,10 @@ __device__ __forceinline__ bool dig_element(const int e, const double* __restric
 #pragma unroll
   for (int t = 0; t < S::NW; ++t) {
     um = max(um, s_max[0][t]);
-    if (VARH1) hm = max(hm, s_max[1][t]);
+    if (VARH1) {
+      hm = max(hm, s_max[1][t]);
+      hl = max(hl, s_max[3][t]);
+    }
   }
   // biased exponent of the largest |u|, one more where its fixed-point form would reach 2^63 (1 - 2^-7)
   const int eu = um ? (int)((um + 0x4000) >> 20) : 1023;
@@ -145,7 +169,7 @@ __device__ __forceinline__ bool dig_element(const int e, const double* __restric
   // exponent of the result's unit before the shift by the derivatives' size (at most 32)
   const int ex = ge + eh + eu - 1023 - kexp - DIG_SH2 - 12;
   if (um >= 0x7ff00000u || hm >= 0x7ff00000u || ge == DIG_BAD || abs(ex) > 800 || abs(ex + e1) > 800 ||
-      abs(eh) > 800 || abs(eu - 1023) > 800) {
+      abs(eh) > 800 || abs(eu - 1023) > 800 || (VARH1 && dig_h1_wide(hm, hl))) {
     const ptrdiff_t at = (ptrdiff_t)e * NP3 + loc;
     dig_fallback<NP, VARH1>(reinterpret_cast<double*>(smem), e, u - at, w - at, G, Df, Dt, h1, h2,
                             VARH1 ? h1L - at : nullptr);

@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(DigEoShape<NP>::T, dig_eo_min_blocks<NP>())
   constexpr int NP2 = NP * NP, NP3 = NP2 * NP;
   if (skip && *skip != 0.0) return;
   extern __shared__ __align__(16) unsigned long long dig_eo_smem[];
-  __shared__ uint32_t s_max[3][S::NW];
+  __shared__ uint32_t s_max[4][S::NW];
   unsigned long long *U = dig_eo_smem, *F = dig_eo_smem + S::FLD;
   const int e = blockIdx.x, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const double* ue = u + (size_t)e * NP3;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(DigEoShape<NP>::T, dig_eo_min_blocks<NP>())
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(Ge), "r"(6 * S::GE * 8) : "memory");
   // the element's exponents
   constexpr int PT = (NP3 + S::T - 1) / S::T;
-  uint32_t um = 0, hm = 0;
+  uint32_t um = 0, hm = 0, hl = 0;
   double uv[PT];
 #pragma unroll
   for (int q = 0; q < PT; ++q) {
@@ -193,25 +193,36 @@ __global__ void __launch_bounds__(DigEoShape<NP>::T, dig_eo_min_blocks<NP>())
 #pragma unroll
   for (int q = 0; q < PT; ++q) um = max(um, (uint32_t)__double2hiint(uv[q]) & 0x7fffffffu);
   if (VARH1)
-    for (int p = threadIdx.x; p < NP3; p += S::T) hm = max(hm, (uint32_t)__double2hiint(he[p]) & 0x7fffffffu);
+    for (int p = threadIdx.x; p < NP3; p += S::T) {
+      const double h = he[p];
+      hm = max(hm, (uint32_t)__double2hiint(h) & 0x7fffffffu);
+      hl = max(hl, dig_h1_low(h));
+    }
   const int ge = gexp[e];
   um = __reduce_max_sync(0xffffffffu, um);
-  if (VARH1) hm = __reduce_max_sync(0xffffffffu, hm);
+  if (VARH1) {
+    hm = __reduce_max_sync(0xffffffffu, hm);
+    hl = __reduce_max_sync(0xffffffffu, hl);
+  }
   if (lane == 0) {
     s_max[0][wp] = um;
     s_max[1][wp] = hm;
+    s_max[3][wp] = hl;
   }
   __syncthreads();
 #pragma unroll
   for (int t = 0; t < S::NW; ++t) {
     um = max(um, s_max[0][t]);
-    if (VARH1) hm = max(hm, s_max[1][t]);
+    if (VARH1) {
+      hm = max(hm, s_max[1][t]);
+      hl = max(hl, s_max[3][t]);
+    }
   }
   const int eu = um ? (int)((um + 0x4000) >> 20) : 1023;
   const int eh = VARH1 ? (hm ? (int)(hm >> 20) - 1022 : 0) : 0;   // |h1| < 2^eh
   const int ex = ge + eh + eu - 1023 - kexp - DIG_SH2 - 12 + 2;   // values and fluxes carry half
   if (um >= 0x7ff00000u || hm >= 0x7ff00000u || ge == DIG_BAD || abs(ex) > 800 || abs(ex + e1) > 800 ||
-      abs(eh) > 800 || abs(eu - 1023) > 800) {
+      abs(eh) > 800 || abs(eu - 1023) > 800 || (VARH1 && dig_h1_wide(hm, hl))) {
     dig_eo_fallback<NP, VARH1>(reinterpret_cast<double*>(dig_eo_smem), e, u, w, G, Df, Dt, h1, h2, h1L);
     return;
   }

@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(DigShape<NP>::T, JAC_MIN_BLOCKS)
   using S = DigShape<NP>;
   constexpr int NP2 = NP * NP, NP3 = NP2 * NP;
   __shared__ __align__(16) unsigned long long smem[S::SMEM];
-  __shared__ uint32_t s_max[3][4];
+  __shared__ uint32_t s_max[4][4];
   __shared__ double s_red[2][4], s_bc[4];
   __shared__ int s_ok;
   if (a.sc[S_DONE] != 0.0) return;
