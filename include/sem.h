@@ -190,7 +190,7 @@ int sem_level_info(const sem_ctx* ctx, int level, sem_level_desc* out);
  * Orders 4 to 11: the FP64 call, and the SEM_AX_PAIRS call at N = 7, 11 and (from 2,048 elements) 9, run in integer
  * digits on the tensor cores (64-bit fixed point per element, any FP64 exponent; the error relative to an element's largest
  * value is below that of FP64 instructions; values of u_L far below their element's largest keep the bits above 2^-62 of it, and
- * an element whose nodal h1_L spans more than 2^8 is computed with FP64 instructions) from a
+ * an element whose nodal h1_L spans more than 2^8 (SEM_AX_PAIRS: 2^13) is computed with FP64 instructions) from a
  * fixed-point copy of the factors that sem_setup builds (48 bytes a point; without the memory for it, and
  * at other orders, FP64 instructions and pairs). Errors: SEM_EINVAL, SEM_ECUDA. */
 int sem_ax(sem_ctx* ctx, const double* u_L, double* w_L, const sem_coef* coef, int flags, void* stream);

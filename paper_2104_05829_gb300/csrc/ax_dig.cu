@@ -37,7 +37,7 @@ namespace sem {
 
 int dig_eo_tables(const Level& L, const int* a, int k, int m2, int q2, DigEoTab** tab, cudaStream_t s);
 const int32_t* dig_eo_exponents(const DigEoTab* tab);
-int ax_dig_eo_apply(const Level& L, int e0, int E, const double* u, double* w, double h1, double h2, const double* h1L,
+int ax_dig_eo_apply(const Level& L, int e0, int E, const double* u, double* w, double h1, double h2, const double* h1L, int span,
                     const double* skip, const EOMat<ArF64>& Df, const EOMat<ArF64>& Dt, cudaStream_t s);
 
 namespace {
@@ -54,13 +54,13 @@ __global__ void __launch_bounds__(DigShape<NP>::T, dig_min_blocks<NP>())
     k_ax_dig(const double* __restrict__ u, double* __restrict__ w, const int2* __restrict__ Gx,
              const int32_t* __restrict__ gexp, const double* __restrict__ G, const DigTab* __restrict__ tab,
              const int kexp, const double h1, const double h2,
-             const double* __restrict__ h1L, const double* skip, const int vec, const int mass, const int e1,
+             const double* __restrict__ h1L, const int span, const double* skip, const int vec, const int mass, const int e1,
              const __grid_constant__ EOMat<ArF64> Df, const __grid_constant__ EOMat<ArF64> Dt) {
   if (skip && *skip != 0.0) return;
   __shared__ __align__(16) unsigned long long smem[DigShape<NP>::SMEM];
   __shared__ uint32_t s_max[4][4];
   double uv[2][2], o[2][2];
-  dig_element<NP, VARH1, false>(blockIdx.x, u, w, Gx, gexp, G, tab, kexp, h1, h2, h1L, vec, mass, e1, Df, Dt, smem,
+  dig_element<NP, VARH1, false>(blockIdx.x, u, w, Gx, gexp, G, tab, kexp, h1, h2, h1L, span, vec, mass, e1, Df, Dt, smem,
                                 s_max, uv, o);
 }
 
@@ -261,7 +261,7 @@ int dig_build(Level& L, cudaStream_t s) {
 
 // The element operator on elements [e0, e0 + E) (u, w, h1L: whole-level L-vectors). Needs L.Gx.
 int ax_dig_apply(const Level& L, int e0, int E, const double* u, double* w, double h1, double h2, const double* h1L,
-                 const double* skip, cudaStream_t s) {
+                 bool pairs, const double* skip, cudaStream_t s) {
   EOMat<ArF64> Df, Dt;
   make_eo<ArF64>(L.D.a, L.NP, false, Df);
   make_eo<ArF64>(L.D.a, L.NP, true, Dt);
@@ -271,7 +271,7 @@ int ax_dig_apply(const Level& L, int e0, int E, const double* u, double* w, doub
   if (h1L) h1L += off;
   const int vec = (((uintptr_t)u | (uintptr_t)w | (uintptr_t)h1L) & 15u) == 0;
   const int mass = h2 != 0.0 ? 1 : 0;                         // h2 B u is added
-  const int e1 = dig_h1_exp(h1);
+  const int e1 = dig_h1_exp(h1), span = dig_h1_span(pairs);
   switch (L.NP) {
 #define CASE(NP)                                                                                                   \
   case NP: {                                                                                                       \
@@ -279,17 +279,17 @@ int ax_dig_apply(const Level& L, int e0, int E, const double* u, double* w, doub
     const int2* Gx = L.Gx + (size_t)e0 * 6 * S::GE;                                                                \
     if (h1L)                                                                                                       \
       k_ax_dig<NP, true><<<E, S::T, 0, s>>>(u, w, Gx, L.gexp + e0, L.G + 7 * off, L.dig, L.dig_kexp, 1.0,   \
-                                            h2, h1L, skip, vec, mass, 0, Df, Dt);                                           \
+                                            h2, h1L, span, skip, vec, mass, 0, Df, Dt);                             \
     else                                                                                                           \
       k_ax_dig<NP, false><<<E, S::T, 0, s>>>(u, w, Gx, L.gexp + e0, L.G + 7 * off, L.dig, L.dig_kexp, h1,   \
-                                             h2, nullptr, skip, vec, mass, e1, Df, Dt);                                      \
+                                             h2, nullptr, 0, skip, vec, mass, e1, Df, Dt);                          \
     SEM_LAUNCH_CHECK();                                                                                            \
     return SEM_OK;                                                                                                 \
   }
     CASE(5) CASE(6) CASE(7) CASE(8)
 #undef CASE
   }
-  if (L.dig_eo) return ax_dig_eo_apply(L, e0, E, u, w, h1, h2, h1L, skip, Df, Dt, s);
+  if (L.dig_eo) return ax_dig_eo_apply(L, e0, E, u, w, h1, h2, h1L, span, skip, Df, Dt, s);
   set_detail("order %d not compiled", L.N);
   return SEM_EINVAL;
 }

@@ -36,16 +36,17 @@ inline __int128 dig_scaled(double x, int num, int den, int s) {
   return neg ? -a : a;
 }
 
-// A nodal h1 is kept in 61 bits below the element's largest, so its values keep FP64's 53 bits down to 2^-8 of that; an element whose
-// h1 spans more (a jump of a material, say) is computed in FP64, which keeps every value's own bits. dig_h1_low is largest for the
-// smallest |h1| that is not zero (a zero is exact in both); dig_h1_wide takes the block's largest high word of |h1| and dig_h1_low.
-constexpr int DIG_H1_SPAN = 61 - 53;
+// A nodal h1 is kept in 61 bits below the element's largest, so its values keep FP64's 53 bits down to 2^-8 of that, and the pairs' 48
+// down to 2^-13; an element whose h1 spans more (a jump of a material, say) is computed in FP64, which keeps every value's own bits.
+// That is slow for a pair call (N = 7, 32^3, every element: 1,555 us against 351 in digits and 448 in pairs). dig_h1_low is largest for
+// the smallest |h1| that is not zero (a zero is exact in both); dig_h1_wide takes the block's largest high word of |h1| and dig_h1_low.
+inline int dig_h1_span(bool pairs) { return 61 - (pairs ? 48 : 53); }
 __device__ __forceinline__ uint32_t dig_h1_low(const double h1) {
   const uint32_t a = (uint32_t)__double2hiint(h1) & 0x7fffffffu;
   return (a | (uint32_t)__double2loint(h1)) ? 0x7fffffffu - a : 0u;
 }
-__device__ __forceinline__ bool dig_h1_wide(const uint32_t high, const uint32_t low) {
-  return (int)(high >> 20) - (int)((0x7fffffffu - low) >> 20) > DIG_H1_SPAN;
+__device__ __forceinline__ bool dig_h1_wide(const uint32_t high, const uint32_t low, const int span) {
+  return (int)(high >> 20) - (int)((0x7fffffffu - low) >> 20) > span;
 }
 
 // exponent of a scalar h1, as the kernel takes it (4096: not a normal number, the elements go to the FP64 form)
@@ -73,7 +74,7 @@ __device__ __forceinline__ bool dig_element(const int e, const double* __restric
                                             const int2* __restrict__ Gx, const int32_t* __restrict__ gexp,
                                             const double* __restrict__ G, const DigTab* __restrict__ tab,
                                             const int kexp, const double h1, const double h2,
-                                            const double* __restrict__ h1L, const int vec, const int mass, const int e1,
+                                            const double* __restrict__ h1L, const int span, const int vec, const int mass, const int e1,
                                             const EOMat<ArF64>& Df, const EOMat<ArF64>& Dt, unsigned long long* smem,
                                             uint32_t (*s_max)[4], double (&uv)[2][2], double (&o)[2][2]) {
   using S = DigShape<NP>;
@@ -169,7 +170,7 @@ __device__ __forceinline__ bool dig_element(const int e, const double* __restric
   // exponent of the result's unit before the shift by the derivatives' size (at most 32)
   const int ex = ge + eh + eu - 1023 - kexp - DIG_SH2 - 12;
   if (um >= 0x7ff00000u || hm >= 0x7ff00000u || ge == DIG_BAD || abs(ex) > 800 || abs(ex + e1) > 800 ||
-      abs(eh) > 800 || abs(eu - 1023) > 800 || (VARH1 && dig_h1_wide(hm, hl))) {
+      abs(eh) > 800 || abs(eu - 1023) > 800 || (VARH1 && dig_h1_wide(hm, hl, span))) {
     const ptrdiff_t at = (ptrdiff_t)e * NP3 + loc;
     dig_fallback<NP, VARH1>(reinterpret_cast<double*>(smem), e, u - at, w - at, G, Df, Dt, h1, h2,
                             VARH1 ? h1L - at : nullptr);

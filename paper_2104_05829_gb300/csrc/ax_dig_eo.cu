@@ -165,8 +165,8 @@ template <int NP, bool VARH1>
 __global__ void __launch_bounds__(DigEoShape<NP>::T, dig_eo_min_blocks<NP>())
     k_ax_dig_eo(const double* __restrict__ u, double* __restrict__ w, const int2* __restrict__ Gx,
                 const int32_t* __restrict__ gexp, const double* __restrict__ G, const DigEoTab* __restrict__ tab,
-                const int kexp, const double h1, const double h2, const double* __restrict__ h1L, const double* skip,
-                const int mass, const int e1, const __grid_constant__ EOMat<ArF64> Df,
+                const int kexp, const double h1, const double h2, const double* __restrict__ h1L, const int span,
+                const double* skip, const int mass, const int e1, const __grid_constant__ EOMat<ArF64> Df,
                 const __grid_constant__ EOMat<ArF64> Dt) {
   using S = DigEoShape<NP>;
   constexpr int NP2 = NP * NP, NP3 = NP2 * NP;
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(DigEoShape<NP>::T, dig_eo_min_blocks<NP>())
   const int eh = VARH1 ? (hm ? (int)(hm >> 20) - 1022 : 0) : 0;   // |h1| < 2^eh
   const int ex = ge + eh + eu - 1023 - kexp - DIG_SH2 - 12 + 2;   // values and fluxes carry half
   if (um >= 0x7ff00000u || hm >= 0x7ff00000u || ge == DIG_BAD || abs(ex) > 800 || abs(ex + e1) > 800 ||
-      abs(eh) > 800 || abs(eu - 1023) > 800 || (VARH1 && dig_h1_wide(hm, hl))) {
+      abs(eh) > 800 || abs(eu - 1023) > 800 || (VARH1 && dig_h1_wide(hm, hl, span))) {
     dig_eo_fallback<NP, VARH1>(reinterpret_cast<double*>(dig_eo_smem), e, u, w, G, Df, Dt, h1, h2, h1L);
     return;
   }
@@ -388,7 +388,7 @@ const int32_t* dig_eo_exponents(const DigEoTab* tab) {
 
 // Elements [e0, e0 + E) of the level; u, w, h1L already at e0.
 int ax_dig_eo_apply(const Level& L, int e0, int E, const double* u, double* w, double h1, double h2, const double* h1L,
-                    const double* skip, const EOMat<ArF64>& Df, const EOMat<ArF64>& Dt, cudaStream_t s) {
+                    int span, const double* skip, const EOMat<ArF64>& Df, const EOMat<ArF64>& Dt, cudaStream_t s) {
   const size_t off = (size_t)e0 * L.NP * L.NP * L.NP;
   const int mass = h2 != 0.0 ? 1 : 0, e1 = dig_h1_exp(h1);
   switch (L.NP) {
@@ -400,12 +400,12 @@ int ax_dig_eo_apply(const Level& L, int e0, int E, const double* u, double* w, d
       SEM_CUDA_TRY(cudaFuncSetAttribute(k_ax_dig_eo<NP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,            \
                                         (int)S::SMEM));                                                                \
       k_ax_dig_eo<NP, true><<<E, S::T, S::SMEM, s>>>(u, w, Gx, L.gexp + e0, L.G + 7 * off, L.dig_eo, L.dig_kexp, 1.0,  \
-                                                     h2, h1L, skip, mass, 0, Df, Dt);                                  \
+                                                     h2, h1L, span, skip, mass, 0, Df, Dt);                            \
     } else {                                                                                                           \
       SEM_CUDA_TRY(cudaFuncSetAttribute(k_ax_dig_eo<NP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
                                         (int)S::SMEM));                                                                \
       k_ax_dig_eo<NP, false><<<E, S::T, S::SMEM, s>>>(u, w, Gx, L.gexp + e0, L.G + 7 * off, L.dig_eo, L.dig_kexp, h1,  \
-                                                      h2, nullptr, skip, mass, e1, Df, Dt);                            \
+                                                      h2, nullptr, 0, skip, mass, e1, Df, Dt);                         \
     }                                                                                                                  \
     SEM_LAUNCH_CHECK();                                                                                                \
     return SEM_OK;                                                                                                     \

@@ -87,7 +87,7 @@ __global__ void k_split_pairs(int64_t n, const double* __restrict__ G, float2* _
 // contractions.
 int ax_eo_apply(const Level& L, const double* u, double* w, double h1, double h2, const double* h1L,
                 const double* skip, cudaStream_t s, bool eo) {
-  if (L.Gx && !eo) return ax_dig_apply(L, 0, L.E, u, w, h1, h2, h1L, skip, s);
+  if (L.Gx && !eo) return ax_dig_apply(L, 0, L.E, u, w, h1, h2, h1L, false, skip, s);
   return eo_launch<ArF64>(L, u, w, L.G, h1, h2, h1L, skip, s);
 }
 
@@ -99,7 +99,7 @@ int ax_pairs_apply(const Level& L, const double* u, double* w, double h1, double
     set_detail("FP32-pair factors were not built");
     return SEM_EINVAL;
   }
-  if (dig_for_pairs(L) && !eo) return ax_dig_apply(L, 0, L.E, u, w, h1, h2, h1L, nullptr, s);
+  if (dig_for_pairs(L) && !eo) return ax_dig_apply(L, 0, L.E, u, w, h1, h2, h1L, true, nullptr, s);
   return eo_launch<ArPair>(L, u, w, L.G2, h1, h2, h1L, nullptr, s);
 }
 
@@ -112,7 +112,7 @@ int ax_eo_apply_range(const Level& L, int e0, int e1, const double* u, double* w
     set_detail("FP32-pair factors not built");
     return SEM_EINVAL;
   }
-  if (pairs ? dig_for_pairs(L) : L.Gx != nullptr) return ax_dig_apply(L, e0, e1 - e0, u, w, h1, h2, h1L, nullptr, s);
+  if (pairs ? dig_for_pairs(L) : L.Gx != nullptr) return ax_dig_apply(L, e0, e1 - e0, u, w, h1, h2, h1L, pairs, nullptr, s);
   const size_t off = (size_t)e0 * L.NP * L.NP * L.NP;
   Level V = L;
   V.E = e1 - e0;

@@ -35,7 +35,7 @@ struct JacArgs {
   int* err;
   long long spin;
   double h1, h2;
-  int kexp, mass, e1, maxit;
+  int kexp, span, mass, e1, maxit;
 };
 
 constexpr int JAC_DIR = INT32_MIN;
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(DigShape<NP>::T, JAC_MIN_BLOCKS)
       for (int x = 0; x < 2; ++x)
         if (has(p, x)) a.p[at + p * NP2 + x] = pv[p][x];
     double o[2][2];
-    const bool held = dig_element<NP, VARH1, true>(e, a.p, a.w, a.Gx, a.gexp, a.G, a.tab, a.kexp, a.h1, a.h2, a.h1L, 0,
+    const bool held = dig_element<NP, VARH1, true>(e, a.p, a.w, a.Gx, a.gexp, a.G, a.tab, a.kexp, a.h1, a.h2, a.h1L, a.span, 0,
                                                    a.mass, a.e1, Df, Dt, smem, s_max, pv, o);
     if (!held) __syncthreads();
     double s1 = 0.0;
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(DigShape<NP>::T, JAC_MIN_BLOCKS)
 // range (N = 7, 8 x 8 x 9 elements: 27.2 against 57.2 us an iteration; N = 4, 5, 6, 8^3: 21.9, 22.4, 25.0 against 43.0, 44.1, 49.1).
 // A spin limit under a millisecond is for callers that test their waits: it keeps the launches, which have none.
 int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, double* w, const double* dinv, double h1,
-                     double h2, const double* h1L, int2* seg, double* sc, int maxit, bool start, cudaStream_t s,
+                     double h2, const double* h1L, bool pairs, int2* seg, double* sc, int maxit, bool start, cudaStream_t s,
                      bool* used) {
   *used = false;
   if (!L.Gx || L.spin_limit < (1ll << 21) || 3 * (int64_t)L.E > 4 * (int64_t)RED_BLOCKS) return SEM_OK;
@@ -334,6 +334,7 @@ int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, do
   a.h1 = h1L ? 1.0 : h1;
   a.h2 = h2;
   a.kexp = L.dig_kexp;
+  a.span = dig_h1_span(pairs);
   a.mass = h2 != 0.0 ? 1 : 0;
   a.e1 = h1L ? 0 : dig_h1_exp(h1);
   a.maxit = maxit;

@@ -266,12 +266,13 @@ int dig_build(Level& L, cudaStream_t s);
 inline bool dig_for_pairs(const Level& L) {
   return L.Gx && (L.NP == 8 || L.NP == 12 || (L.NP == 10 && L.E >= 2048));
 }
+// pairs: an FP32-pair call (which span of a nodal h1 stays in digits)
 int ax_dig_apply(const Level& L, int e0, int E, const double* u, double* w, double h1, double h2, const double* h1L,
-                 const double* skip, cudaStream_t s);
+                 bool pairs, const double* skip, cudaStream_t s);
 
 // ---- jacobi_dig.cu: iterations of a small mesh's Jacobi-PCG in one cooperative launch (digit operator)
 int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, double* w, const double* dinv, double h1,
-                     double h2, const double* h1L, int2* seg, double* sc, int maxit, bool start, cudaStream_t s,
+                     double h2, const double* h1L, bool pairs, int2* seg, double* sc, int maxit, bool start, cudaStream_t s,
                      bool* used);
 
 // ---- ax_eo.cu (FP32-pair variant)

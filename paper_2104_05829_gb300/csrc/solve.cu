@@ -811,7 +811,8 @@ int solve_impl(Ctx* C, Proj* P, const double* f, const sem_coef* c, double tol, 
       }
       if (one) {
         const int nb = std::min(1024, maxit - launched);
-        SEM_TRY(jacobi_dig_solve(*C, L, u, C->r, C->p, w, dinv, c->h1, c->h2, c->h1_L, reinterpret_cast<int2*>(C->t), sc,
+        SEM_TRY(jacobi_dig_solve(*C, L, u, C->r, C->p, w, dinv, c->h1, c->h2, c->h1_L, pairs,
+                                 reinterpret_cast<int2*>(C->t), sc,
                                  nb, launched == 0, s, &one));
         if (one) {
           launched += nb;

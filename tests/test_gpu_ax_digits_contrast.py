@@ -57,3 +57,23 @@ def test_one_launch_solve_with_elements_of_the_fp64_form(low):
     assert np.abs(xa - xb).max() <= 30 * 4e5 ** 0.5 * 2.0 ** -53 * 1e2 / low * np.abs(xb).max()
     one.close()
     chain.close()
+
+
+@pytest.mark.parametrize("N", [7, 11])
+def test_pair_calls_keep_48_bits_of_small_values(N):
+    """h1 spans 2^12 and a little: within what a pair call leaves in digits."""
+    mesh = si.box_mesh((3, 2, 2), N, warp=0.1, perm_seed=1)
+    ctx = ctx_for(mesh, prec_copies=4)
+    u = T(si.uniform_field(mesh, 3, continuous=False))
+    low = 2.0 ** -12
+    edge = np.zeros((N + 1,) * 3, dtype=bool)
+    edge[0, 0, :] = True
+    ramp = np.broadcast_to(1.0 + np.arange(N + 1) / (2.0 * N + 2.0), mesh["x"].shape)   # 1 to 1.5: one binade
+    h1 = T(np.where(edge, ramp, low * ramp))
+    ref, w = (H(ctx.ax(u, h1_L=h1, assemble=False, pairs=p)).reshape(mesh["x"].shape) for p in (False, True))
+    for e in range(mesh["E"]):
+        # the terms' 2^-48, as for FP64's 2^-53 above
+        assert relmax(w[e, 1:, 1:], ref[e, 1:, 1:]) < 6 * 12 * 2.0 ** -48 * 8 * 1.5
+    # a pair call takes the digits there, the FP64 call the FP64 form
+    assert not np.array_equal(w, ref)
+    ctx.close()
