@@ -373,7 +373,7 @@ int advect_apply(Ctx& C, int prec, const void* c, const void* u, void* w, int nc
   if (prec != SEM_FP32) {
     SEM_TRY(advect_dig_build(A, L, s));
     // at N = 4 (lines and outputs padded from five and eight points) the pair form is the faster one
-    if (A.Gqx && (prec == SEM_FP64 || L.N >= 5)) return advect_dig_apply(L, A, (const double*)c, (const double*)u, (double*)w, ncomp, s);
+    if (A.Gqx && (prec == SEM_FP64 || L.N >= 5)) return advect_dig_apply(L, A, (const double*)c, (const double*)u, (double*)w, ncomp, prec == SEM_FP64P, s);
   }
   if (prec == SEM_FP64P) {
     SEM_TRY(advect_pairs_build(A, L, s));

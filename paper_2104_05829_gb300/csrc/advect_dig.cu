@@ -33,6 +33,13 @@ namespace sem {
 namespace {
 
 constexpr int ADV_SH = 48;
+// The factors and the wind have one exponent each, so where chat comes out 2^-k of what the two could give, it keeps 61 - k bits: the
+// wind along a thin element, with one large and one small component and the metric the other way round. FP64 keeps every
+// product's own bits. Elements that lose more than these go to the FP64 form (53 bits, less the one that a bound may be off; 48).
+// Smooth data, elements 2^-k of their width thick, 2-norm error against 128-bit arithmetic at k = 0, 6, 8, 10, 14, 20: N = 7 2.5e-15, 2.4e-15,
+// 2.9e-15, 9.5e-15, 1.5e-13, 9.9e-12 in digits throughout and at most 3.9e-15, the FP64 form's at any k, with the line here
+// (N = 4: up to 1.0e-11, and 3.3e-15). What it costs a call without such elements: nothing (24^3, N = 7: 2.84 ms before and after).
+constexpr int ADV_LOSS = 61 - 53 - 1, ADV_LOSS_PAIRS = 61 - 48;
 
 template <int NP>
 struct DigAdv {
@@ -131,7 +138,7 @@ template <int NP>
 __global__ void __launch_bounds__(DigAdv<NP>::T, 2)
     k_advect_dig(const int ncomp, const int64_t nL, const double* __restrict__ cv, const double* __restrict__ uv,
                  const int2* __restrict__ Gx, const int32_t* __restrict__ gexp, const AdvDigTab* __restrict__ tab,
-                 const int ebase, double* __restrict__ wv, const double* __restrict__ Gq, const double* __restrict__ Im,
+                 const int ebase, const int loss, double* __restrict__ wv, const double* __restrict__ Gq, const double* __restrict__ Im,
                  const double* __restrict__ Dq, const __grid_constant__ AdvOps<double, NP> P) {
   using S = DigAdv<NP>;
   constexpr int NQ = S::NQ, NP2 = S::NP2, NP3 = S::NP3, W = S::W, LQ = S::LQ;
@@ -281,6 +288,7 @@ __global__ void __launch_bounds__(DigAdv<NP>::T, 2)
       }
     });
     sc = s1 + s2;
+    bad = s2 > loss && cm != 0;
   }
 
   // 3. every advected component
@@ -689,7 +697,8 @@ int advect_dig_build(AdvData& A, const Level& L, cudaStream_t s) {
 }
 
 int advect_dig_apply(const Level& L, const AdvData& A, const double* c, const double* u, double* w, int ncomp,
-                     cudaStream_t s) {
+                     bool pairs, cudaStream_t s) {
+  const int loss = pairs ? ADV_LOSS_PAIRS : ADV_LOSS;
   switch (L.NP) {
 #define CASE(NP)                                                                                                      \
   case NP: {                                                                                                          \
@@ -697,8 +706,8 @@ int advect_dig_apply(const Level& L, const AdvData& A, const double* c, const do
     constexpr size_t smem = std::max(S::SMEM, advect_smem<AdvPlain<double>, NP>());                                   \
     static PerDevice<bool> attr;                                                                                      \
     SEM_TRY(smem_attr_once(attr, (const void*)k_advect_dig<NP>, smem));                                               \
-    k_advect_dig<NP><<<L.E, S::T, smem, s>>>(ncomp, L.nL, c, u, A.Gqx, A.gqexp, A.dig, A.dig_ebase, w, A.Gq, A.Im,     \
-                                             A.Dq, adv_ops<AdvPlain<double>, NP>(A));                                 \
+    k_advect_dig<NP><<<L.E, S::T, smem, s>>>(ncomp, L.nL, c, u, A.Gqx, A.gqexp, A.dig, A.dig_ebase, loss, w, A.Gq,     \
+                                             A.Im, A.Dq, adv_ops<AdvPlain<double>, NP>(A));                           \
     SEM_LAUNCH_CHECK();                                                                                               \
     return SEM_OK;                                                                                                    \
   }

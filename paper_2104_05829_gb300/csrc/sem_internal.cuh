@@ -349,7 +349,7 @@ int char_advance(Ctx& C, int prec, const void* c0, const void* c1, void* w, int 
 // ---- advect_dig.cu: the same in integer digits (FP64 data)
 int advect_dig_build(AdvData& A, const Level& L, cudaStream_t s);
 int advect_dig_apply(const Level& L, const AdvData& A, const double* c, const double* u, double* w, int ncomp,
-                     cudaStream_t s);
+                     bool pairs, cudaStream_t s);   // pairs: an FP32-pair call
 
 // ---- proj.cu: projection of successive right-hand sides
 struct Proj;
