@@ -150,13 +150,15 @@ __global__ void __launch_bounds__(DigAdv<NP>::T, 2)
   const int g = lane >> 2, c = lane & 3;
   const size_t eb = (size_t)e * NP3;
   const DigStart zs;
-  // largest |value| of n fields (high words) over the element; one barrier
+  // largest |value| of n fields (high words, at least 1 for a value that is not zero) over the element; one barrier
   int par = 0;
   auto largest = [&](const double* v, int n) {
     uint32_t m = 0;
     for (int f = 0; f < n; ++f)
-      for (int q = threadIdx.x; q < NP3; q += S::T)
-        m = max(m, (uint32_t)__double2hiint(v[(size_t)f * nL + eb + q]) & 0x7fffffffu);
+      for (int q = threadIdx.x; q < NP3; q += S::T) {
+        const double x = v[(size_t)f * nL + eb + q];
+        m = max(m, ((uint32_t)__double2hiint(x) & 0x7fffffffu) | (__double2loint(x) != 0));
+      }
     m = __reduce_max_sync(0xffffffffu, m);
     if (lane == 0) s_max[par][wp] = m;
     __syncthreads();

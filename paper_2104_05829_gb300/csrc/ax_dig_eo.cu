@@ -151,17 +151,6 @@ __device__ __forceinline__ uint32_t dig_eo_pass(const unsigned long long* U, uns
 }
 
 template <int NP, bool VARH1>
-__device__ __noinline__ void dig_eo_fallback(double* A, int e, const double* u, double* w, const double* G,
-                                             const EOMat<ArF64>& Df, const EOMat<ArF64>& Dt, double h1, double h2,
-                                             const double* h1L) {
-  constexpr int NP2 = NP * NP;
-  const bool on = threadIdx.x < NP2;
-  const int ij = on ? threadIdx.x : 0;
-  eo_element<ArF64, NP, VARH1>(on, on, ij % NP, ij / NP, (size_t)e * NP2 * NP, u, w, G + (size_t)e * 7 * NP2 * NP, Df,
-                               Dt, h1, h2, h1L, A, A + Pad3<NP>::ES, A + 2 * Pad3<NP>::ES);
-}
-
-template <int NP, bool VARH1>
 __global__ void __launch_bounds__(DigEoShape<NP>::T, dig_eo_min_blocks<NP>())
     k_ax_dig_eo(const double* __restrict__ u, double* __restrict__ w, const int2* __restrict__ Gx,
                 const int32_t* __restrict__ gexp, const double* __restrict__ G, const DigEoTab* __restrict__ tab,
@@ -221,9 +210,10 @@ __global__ void __launch_bounds__(DigEoShape<NP>::T, dig_eo_min_blocks<NP>())
   const int eu = um ? (int)((um + 0x4000) >> 20) : 1023;
   const int eh = VARH1 ? (hm ? (int)(hm >> 20) - 1022 : 0) : 0;   // |h1| < 2^eh
   const int ex = ge + eh + eu - 1023 - kexp - DIG_SH2 - 12 + 2;   // values and fluxes carry half
-  if (um >= 0x7ff00000u || hm >= 0x7ff00000u || ge == DIG_BAD || abs(ex) > 800 || abs(ex + e1) > 800 ||
-      abs(eh) > 800 || abs(eu - 1023) > 800 || (VARH1 && dig_h1_wide(hm, hl, span))) {
-    dig_eo_fallback<NP, VARH1>(reinterpret_cast<double*>(dig_eo_smem), e, u, w, G, Df, Dt, h1, h2, h1L);
+  const bool off = hm >= 0x7ff00000u || ge == DIG_BAD || abs(ex) > 800 || abs(ex + e1) > 800 || abs(eh) > 800 ||
+                   abs(eu - 1023) > 800 || (VARH1 && dig_h1_wide(hm, hl, span));
+  if (um - 1u >= 0x7fefffffu || off) {   // um zero, or that of an Inf or NaN
+    dig_fallback<NP, VARH1>(reinterpret_cast<double*>(dig_eo_smem), e, u, w, G, Df, Dt, h1, h2, h1L, !off && um == 0);
     return;
   }
 #pragma unroll
