@@ -163,29 +163,30 @@ __global__ void __launch_bounds__(DigShape<NP>::T, JAC_MIN_BLOCKS)
 #pragma unroll
       for (int x = 0; x < 2; ++x) {
         const int2 sg = has(p, x) ? a.seg[at + p * NP2 + x] : make_int2(0, 0);
-        if (sg.y == JAC_DIR) o[p][x] = 0.0;
-        if (sg.y <= 0) continue;
-        if (sg.y <= 8) {
-          double v[8];
+        const int few = sg.y <= 8 ? sg.y : 0;
+        double v[8];
 #pragma unroll
-          for (int t = 0; t < 8; ++t) v[t] = t < sg.y ? __ldcg(a.w + a.idx[sg.x + t]) : 0.0;
-          const int most = __reduce_max_sync(__activemask(), sg.y);   // fewer FP64 instructions where no lane needs them
+        for (int t = 0; t < 8; ++t) v[t] = t < few ? __ldcg(a.w + a.idx[sg.x + t]) : 0.0;
+        const int most = __reduce_max_sync(0xffffffffu, few);   // fewer FP64 instructions where no lane needs them
+        if (few > 0) {
           double t1 = v[0] + v[1];
           if (most > 2) {
 #pragma unroll
             for (int t = 2; t < 4; ++t)
-              if (t < sg.y) t1 += v[t];
+              if (t < few) t1 += v[t];
             if (most > 4) {
 #pragma unroll
               for (int t = 4; t < 8; ++t)
-                if (t < sg.y) t1 += v[t];
+                if (t < few) t1 += v[t];
             }
           }
           o[p][x] = t1;
-        } else {
+        } else if (sg.y > 8) {
           double t1 = __ldcg(a.w + a.idx[sg.x]);
           for (int t = 1; t < sg.y; ++t) t1 += __ldcg(a.w + a.idx[sg.x + t]);
           o[p][x] = t1;
+        } else if (sg.y == JAC_DIR) {
+          o[p][x] = 0.0;
         }
       }
     __syncthreads();
