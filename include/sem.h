@@ -26,6 +26,8 @@
  * sem_free; sem_ax, sem_gs and the level operators allocate nothing.
  * `stream` is a cudaStream_t passed as void* (NULL = legacy default stream);
  * calls are asynchronous on it except where noted.
+ * A context's calls share its workspaces and the scratch of its reductions: order them, by one stream or by events
+ * between streams. Contexts are independent.
  *
  * Errors. Every int-returning call returns SEM_OK (0) or a negative code
  * below; sem_strerror gives a message and sem_last_error_detail the last

@@ -289,7 +289,7 @@ int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, do
                      double h2, const double* h1L, bool pairs, int2* seg, double* sc, int maxit, bool start, cudaStream_t s,
                      bool* used) {
   *used = false;
-  if (!L.Gx || L.spin_limit < (1ll << 21) || 3 * (int64_t)L.E > 4 * (int64_t)RED_BLOCKS) return SEM_OK;
+  if (!L.Gx || L.spin_limit < (1ll << 21) || L.E > JAC_MAX_E) return SEM_OK;
   int dev = 0, nsm = 0, coop = 0, per_sm = 0;
   SEM_CUDA_TRY(cudaGetDevice(&dev));
   SEM_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -326,9 +326,9 @@ int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, do
   a.own = L.owner;
   a.seg = seg;
   a.idx = L.seg_idx;
-  a.part = C.red_part;
+  a.part = C.jac;
   a.sc = sc;
-  unsigned* sync = reinterpret_cast<unsigned*>(C.scal + 4 * S_NSLOTS);   // its own slot set
+  unsigned* sync = reinterpret_cast<unsigned*>(C.jac + 3 * JAC_MAX_E);
   a.bar = sync;
   a.err = reinterpret_cast<int*>(sync + 1);
   a.spin = L.spin_limit;

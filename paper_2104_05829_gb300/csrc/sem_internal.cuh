@@ -204,7 +204,9 @@ struct Ctx {
   // deterministic reduction scratch
   double* red_part = nullptr;       // [RED_BLOCKS * 4]
   unsigned int* red_ticket = nullptr;
-  double* scal = nullptr;           // [5 * S_NSLOTS]: outer, coarse, sem_dot, Lanczos, one-launch Jacobi-PCG
+  double* scal = nullptr;           // [4 * S_NSLOTS]: outer, coarse, sem_dot, Lanczos
+  double* jac = nullptr;            // [3 * JAC_MAX_E + 1]: block parts and barrier words of the one-launch Jacobi-PCG, which is
+                                    // under way for up to 1,024 iterations: not shared with the reductions
   double* h_scal = nullptr;         // pinned mirror
   // fine-level FP64 solver workspace
   double *r = nullptr, *z = nullptr, *p = nullptr, *w = nullptr, *t = nullptr;
@@ -236,6 +238,7 @@ struct Ctx {
 // the narrow FP64 pipe); fixed for determinism
 constexpr int RED_BLOCKS = 1216;
 constexpr int RED_THREADS = 256;
+constexpr int JAC_MAX_E = 1024;   // elements of the one-launch Jacobi-PCG at most (four blocks on each of 152 SMs: 608)
 
 // ---- ax.cu
 // eo: the FP64 operator in its even-odd FP64 (or FP32-pair) form, not in digits

@@ -385,7 +385,7 @@ void sem_free(sem_ctx* h) {
   if (!C) return;
   for (int l = 0; l < SEM_MAX_LEVELS; ++l) free_level(C->lev[l]);
   advect_free(C->adv);
-  void* ptrs[] = {C->red_part, C->red_ticket, C->scal, C->r, C->z, C->p, C->w, C->t,
+  void* ptrs[] = {C->red_part, C->red_ticket, C->scal, C->jac, C->r, C->z, C->p, C->w, C->t,
                   C->cg_err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -506,8 +506,9 @@ int sem_setup(const sem_mesh* m, const sem_opts* opts_in, sem_ctx** out) {
   STEP(dmalloc(&C->red_ticket, 1));
   STEP(dmalloc(&C->cg_err, 1));
   CUSTEP(cudaMemsetAsync(C->red_ticket, 0, sizeof(unsigned), s));
-  STEP(dmalloc(&C->scal, 5 * S_NSLOTS));
-  CUSTEP(cudaMemsetAsync(C->scal, 0, 5 * S_NSLOTS * sizeof(double), s));
+  STEP(dmalloc(&C->scal, 4 * S_NSLOTS));
+  CUSTEP(cudaMemsetAsync(C->scal, 0, 4 * S_NSLOTS * sizeof(double), s));
+  STEP(dmalloc(&C->jac, 3 * JAC_MAX_E + 1));
   CUSTEP(cudaMallocHost((void**)&C->h_scal, 4 * S_NSLOTS * sizeof(double)));
   STEP(dmalloc(&C->r, nL));
   STEP(dmalloc(&C->z, nL));
