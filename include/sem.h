@@ -125,9 +125,9 @@ typedef struct {
   int32_t coarse_mode;       /* how the order-1 coarse Jacobi-PCG runs: SEM_COARSE_* (default AUTO) */
   int64_t spin_limit;        /* SM clock cycles a device-side wait may spin before it gives up (2^31, about a
                                 second at GB300's clock; >= 0). A wait that gives up makes the solve that
-                                launched it return SEM_EBREAKDOWN (the coarse solve's exchange waits, the grid
-                                barriers of a small Jacobi-PCG; limits below 2^21 keep that solve to kernels
-                                without waits) or turns
+                                launched it return SEM_EBREAKDOWN (the coarse solve's exchange waits), go on from
+                                its last result with kernels without waits (the grid barriers of a small
+                                Jacobi-PCG; limits from 1 to 2^21 - 1 keep it to those from the start) or turns
                                 the outputs of the waiting block into NaN (the FP32 operator's bulk-copy wait,
                                 which then waits once more, with the default limit, for its copies to land) */
 } sem_opts;

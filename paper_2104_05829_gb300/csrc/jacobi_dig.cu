@@ -9,7 +9,8 @@
 //   2. x, r updated; the element's parts of (r, r) and (r, D^-1 r), stored;
 //   barrier; beta, p.
 // Every block adds all the parts in the same fixed order, so all take the same alpha and beta and leave in the same
-// iteration. A wait is bounded (sem_opts.spin_limit); when one gives up, all blocks leave and the solve reports a breakdown.
+// iteration. A wait is bounded (sem_opts.spin_limit). x, r and the scalars are written only once all blocks are through (jac_commit); when
+// a wait gives up, all blocks leave without a write to them, and the kernels without waits take the solve over from there.
 // Measured, an iteration: N = 7, one element 32.8 -> 11.0 us, 4^3 36.9 -> 14.4, 6^3 42.5 -> 17.9, 8^3 55.0 -> 25.3 (the manufactured
 // 4^3 solve 6.9 -> 2.8 ms). What is left at one element is latency: the operator's chain, two barriers and four
 // reductions; at four elements an SM the FP64 instructions of the vector work (about 400 a block, 16 cycles each), so sums
@@ -31,14 +32,15 @@ struct JacArgs {
   const int2* seg;       // per point: position of its node's copies in idx, count (0: the only copy); Dirichlet: bit 31
   const int32_t* idx;
   double *part, *sc;
-  unsigned* bar;         // arrivals so far
-  int* err;
+  unsigned* bar;         // arrivals so far; then blocks that are through
+  int* state;            // 0: under way, JAC_GIVEN_UP, JAC_THROUGH
   long long spin;
   double h1, h2;
   int kexp, span, mass, e1, maxit;
 };
 
 constexpr int JAC_DIR = INT32_MIN;
+constexpr int JAC_GIVEN_UP = 1, JAC_THROUGH = 2;
 
 // Blocks an SM: registers for the vectors next to the operator's.
 constexpr int JAC_MIN_BLOCKS = 4;
@@ -60,11 +62,21 @@ __device__ __forceinline__ bool jac_arrive_wait(const JacArgs& a, unsigned targe
   while (true) {
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.bar) : "memory");
     if ((int)(v - target) >= 0) return true;
-    if ((++polls & 63u) == 0) {
-      if (clock64() - t0 > a.spin) atomicExch(a.err, 1);
-      if (*(volatile int*)a.err != 0) return false;
-    }
+    const bool late = clock64() - t0 > a.spin;
+    if (late) atomicCAS(a.state, 0, JAC_GIVEN_UP);
+    if ((late || (++polls & 63u) == 0) && *(volatile int*)a.state != 0) return false;
   }
+}
+
+// Whether this launch's result counts, the same answer in every block (one thread each): `state` leaves 0 once, to JAC_THROUGH by
+// the last block that is through its iterations, to JAC_GIVEN_UP by the first wait that gives up, here or at a barrier.
+__device__ __forceinline__ bool jac_commit(const JacArgs& a, unsigned* through, unsigned E) {
+  if (atomicAdd(through, 1u) == E - 1) atomicCAS(a.state, 0, JAC_THROUGH);
+  const long long t0 = clock64();
+  int v;
+  while ((v = *(volatile int*)a.state) == 0)
+    if (clock64() - t0 > a.spin) atomicCAS(a.state, 0, JAC_GIVEN_UP);
+  return v == JAC_THROUGH;
 }
 
 __device__ __forceinline__ double jac_warp_sum(double v) {
@@ -254,6 +266,10 @@ __global__ void __launch_bounds__(DigShape<NP>::T, JAC_MIN_BLOCKS)
 #pragma unroll
       for (int x = 0; x < 2; ++x) pv[p][x] = fma(beta, pv[p][x], zv[p][x]);
   }
+  if (!ok) return;
+  if (threadIdx.x == 0) s_ok = jac_commit(a, a.bar + 2, E);
+  __syncthreads();
+  if (!s_ok) return;
 #pragma unroll
   for (int p = 0; p < 2; ++p)
 #pragma unroll
@@ -272,24 +288,26 @@ __global__ void __launch_bounds__(DigShape<NP>::T, JAC_MIN_BLOCKS)
     a.sc[S_RR] = rr;
     a.sc[S_ITER] += it;
     a.sc[S_TOTAL] += it;
-    if (bad || !ok) a.sc[S_BREAK] = 1.0;
-    if (bad || !ok || done) a.sc[S_DONE] = 1.0;
+    if (bad) a.sc[S_BREAK] = 1.0;
+    if (bad || done) a.sc[S_DONE] = 1.0;
   }
 }
 
 }  // namespace
 
-// Iterations of a started Jacobi-PCG (pcg_begin_tol), at most maxit of them, in one cooperative launch, where the mesh's
-// blocks fit on the device together. seg: room for 2 nL 32-bit words. *used: false when the solve takes the launches.
+// Iterations of a started Jacobi-PCG (pcg_begin_tol), at most maxit >= 1 of them, in one cooperative launch, where the mesh's
+// blocks fit on the device together. seg: room for 2 nL 32-bit words. *used: false when the solve takes the launches. A launch whose
+// waits gave up leaves x, r and the scalars as they were (S_ITER and S_DONE tell) and p undefined: jacobi_dig_resume makes it D^-1 r.
 //
 // The rule. All blocks must be resident, four on an SM: up to 608 elements on 152 SMs. It is the faster form over that whole
 // range (N = 7, 8 x 8 x 9 elements: 27.2 against 57.2 us an iteration; N = 4, 5, 6, 8^3: 21.9, 22.4, 25.0 against 43.0, 44.1, 49.1).
-// A spin limit under a millisecond is for callers that test their waits: it keeps the launches, which have none.
+// A spin limit under a millisecond could run out in an ordinary solve: it keeps the launches, which have no waits. A limit of
+// zero does not: every barrier gives up at the first poll that finds a block missing, and the launches take over.
 int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, double* w, const double* dinv, double h1,
                      double h2, const double* h1L, bool pairs, int2* seg, double* sc, int maxit, bool start, cudaStream_t s,
                      bool* used) {
   *used = false;
-  if (!L.Gx || L.spin_limit < (1ll << 21) || L.E > JAC_MAX_E) return SEM_OK;
+  if (!L.Gx || (L.spin_limit != 0 && L.spin_limit < (1ll << 21)) || L.E > JAC_MAX_E) return SEM_OK;
   int dev = 0, nsm = 0, coop = 0, per_sm = 0;
   SEM_CUDA_TRY(cudaGetDevice(&dev));
   SEM_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -330,7 +348,7 @@ int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, do
   a.sc = sc;
   unsigned* sync = reinterpret_cast<unsigned*>(C.jac + 3 * JAC_MAX_E);
   a.bar = sync;
-  a.err = reinterpret_cast<int*>(sync + 1);
+  a.state = reinterpret_cast<int*>(sync + 1);
   a.spin = L.spin_limit;
   a.h1 = h1L ? 1.0 : h1;
   a.h2 = h2;
@@ -348,7 +366,7 @@ int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, do
       k_jac_seg<<<(unsigned)((L.n_seg + 255) / 256), 256, 0, s>>>(L.n_seg, L.seg_off, L.seg_idx, L.seg_dir, seg);
     SEM_LAUNCH_CHECK();
   }
-  SEM_CUDA_TRY(cudaMemsetAsync(sync, 0, 2 * sizeof(unsigned), s));
+  SEM_CUDA_TRY(cudaMemsetAsync(sync, 0, 3 * sizeof(unsigned), s));
   void* args[] = {&a, &Df, &Dt};
   const cudaError_t rc = cudaLaunchCooperativeKernel(f, dim3(L.E), dim3(threads), args, 0, s);
   if (rc == cudaErrorCooperativeLaunchTooLarge) {   // a part of the device only (MPS, green contexts): the launches
@@ -358,6 +376,13 @@ int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, do
   SEM_CUDA_TRY(rc);
   *used = true;
   return SEM_OK;
+}
+
+// p = D^-1 r, the start of the iteration from x and r, after a launch that gave up.
+int jacobi_dig_resume(const Level& L, double* p, const double* r, const double* dinv, double* sc, cudaStream_t s) {
+  SEM_CUDA_TRY(cudaMemsetAsync(p, 0, (size_t)L.nL * sizeof(double), s));
+  SEM_CUDA_TRY(cudaMemsetAsync(sc + S_BETA, 0, sizeof(double), s));
+  return kr_direction_jacobi(L, SEM_FP64, p, r, dinv, sc, s);   // D^-1 r + beta 0
 }
 
 }  // namespace sem

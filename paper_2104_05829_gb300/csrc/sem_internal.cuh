@@ -205,7 +205,7 @@ struct Ctx {
   double* red_part = nullptr;       // [RED_BLOCKS * 4]
   unsigned int* red_ticket = nullptr;
   double* scal = nullptr;           // [4 * S_NSLOTS]: outer, coarse, sem_dot, Lanczos
-  double* jac = nullptr;            // [3 * JAC_MAX_E + 1]: block parts and barrier words of the one-launch Jacobi-PCG, which is
+  double* jac = nullptr;            // [3 * JAC_MAX_E + 2]: block parts and barrier words of the one-launch Jacobi-PCG, which is
                                     // under way for up to 1,024 iterations: not shared with the reductions
   double* h_scal = nullptr;         // pinned mirror
   // fine-level FP64 solver workspace
@@ -277,6 +277,7 @@ int ax_dig_apply(const Level& L, int e0, int E, const double* u, double* w, doub
 int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, double* w, const double* dinv, double h1,
                      double h2, const double* h1L, bool pairs, int2* seg, double* sc, int maxit, bool start, cudaStream_t s,
                      bool* used);
+int jacobi_dig_resume(const Level& L, double* p, const double* r, const double* dinv, double* sc, cudaStream_t s);
 
 // ---- ax_eo.cu (FP32-pair variant)
 int pairs_build(Level& L, cudaStream_t s);

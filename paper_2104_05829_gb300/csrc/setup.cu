@@ -508,7 +508,7 @@ int sem_setup(const sem_mesh* m, const sem_opts* opts_in, sem_ctx** out) {
   CUSTEP(cudaMemsetAsync(C->red_ticket, 0, sizeof(unsigned), s));
   STEP(dmalloc(&C->scal, 4 * S_NSLOTS));
   CUSTEP(cudaMemsetAsync(C->scal, 0, 4 * S_NSLOTS * sizeof(double), s));
-  STEP(dmalloc(&C->jac, 3 * JAC_MAX_E + 1));
+  STEP(dmalloc(&C->jac, 3 * JAC_MAX_E + 2));
   CUSTEP(cudaMallocHost((void**)&C->h_scal, 4 * S_NSLOTS * sizeof(double)));
   STEP(dmalloc(&C->r, nL));
   STEP(dmalloc(&C->z, nL));

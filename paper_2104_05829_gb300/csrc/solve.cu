@@ -793,12 +793,18 @@ int solve_impl(Ctx* C, Proj* P, const double* f, const sem_coef* c, double tol, 
     const int batch = 8;
     // the one-launch form (b is read no more: its array holds the points' copies), at most 1,024 iterations a launch
     bool one = pairs ? dig_for_pairs(L) : L.Gx != nullptr;
-    int launched = 0;
+    int launched = 0, in_one = 0;   // in_one: iterations of the one-launch form that was launched last
     while (true) {
       SEM_TRY(read_scalars(*C, 0, s));
       const double* hs = C->h_scal;
       bb = hs[S_BB];
       rr = hs[S_RR];
+      if (in_one && hs[S_DONE] == 0.0 && (int)hs[S_ITER] == iters) {   // its waits gave up
+        one = false;
+        launched -= in_one;
+        SEM_TRY(jacobi_dig_resume(L, C->p, C->r, dinv, sc, s));
+      }
+      in_one = 0;
       iters = (int)hs[S_ITER];
       if (hs[S_BREAK] != 0.0) {
         rc = SEM_EBREAKDOWN;
@@ -816,6 +822,7 @@ int solve_impl(Ctx* C, Proj* P, const double* f, const sem_coef* c, double tol, 
                                  nb, launched == 0, s, &one));
         if (one) {
           launched += nb;
+          in_one = nb;
           continue;
         }
       }
