@@ -193,7 +193,7 @@ int sem_level_info(const sem_ctx* ctx, int level, sem_level_desc* out);
  * digits on the tensor cores (64-bit fixed point per element, any FP64 exponent; the error relative to an element's largest
  * value is below that of FP64 instructions; values of u_L far below their element's largest keep the bits above 2^-62 of it, and
  * an element whose nodal h1_L spans more than 2^8 (SEM_AX_PAIRS: 2^13) is computed with FP64 instructions) from a
- * fixed-point copy of the factors that sem_setup builds (48 bytes a point; without the memory for it, and
+ * fixed-point copy of the factors that sem_setup builds (48 bytes a point, 58 at N = 4; without the memory for it, and
  * at other orders, FP64 instructions and pairs). Errors: SEM_EINVAL, SEM_ECUDA. */
 int sem_ax(sem_ctx* ctx, const double* u_L, double* w_L, const sem_coef* coef, int flags, void* stream);
 
@@ -266,7 +266,10 @@ int sem_get_lmax(const sem_ctx* ctx, double* lmax, int n);
  * smoother and levels run in `prec` (SEM_FP64, SEM_FP32, SEM_BF16G); the
  * outer iteration, residual and dot products are always FP64. A nodal
  * coef->h1_L works with both (p-MG: CHEBY-JAC, see sem_precond_setup_nodal) and
- * with SEM_OUTER_PAIRS. f_L: nodal
+ * with SEM_OUTER_PAIRS. The outer operator is sem_ax's (in digits at N = 4..11), except with a SEM_FP32 or SEM_BF16G
+ * V-cycle and tol > 1e-9: there, and in sem_proj_update and the eigenvalue estimates of a scalar h1, FP64 instructions (or the
+ * FP32-pair kernel) run, so that results stay bit for bit what they were without digits; such solves should ask for
+ * SEM_OUTER_PAIRS (24^3 elements, N = 7, FP32 CHEBY-JAC to 1e-8: 24.5 ms without it, 16.9 with). f_L: nodal
  * function or assembled b (rhs_flags). u_L: solution (continuous L-vector).
  * Blocks until done (reads one residual norm per iteration). Errors:
  * SEM_ENOTCONV (info filled, u_L holds the last iterate), SEM_EBREAKDOWN,
@@ -326,7 +329,9 @@ int sem_solve_proj(sem_ctx* ctx, sem_proj* pj, const double* f_L, const sem_coef
  * cubature factors, 9 nq^3 float2 per element, are built on the first such call) or SEM_FP32
  * (float vectors, FP32 arithmetic). SEM_FP64 at N = 4..7 and SEM_FP64P at N = 5..7 run in integer digits on the
  * tensor cores, from a fixed-point copy of the cubature factors (9 nq^3 64-bit values per element, built on the
- * first such call; without the memory for it, as at the other orders).
+ * first such call; without the memory for it, as at the other orders; elements whose contravariant wind is below 2^-7
+ * (SEM_FP64P: 2^-13) of what their metric and c_L could give, thin elements with the wind along them, are computed with FP64
+ * instructions).
  * The cubature factors w J dr/dx at the Gauss points are built on the first call
  * (synchronous; 9 nq^3 values per element in FP64 and FP32). Compiled for 2 <= N <= 8. */
 #define SEM_ADV_LOCAL 0

@@ -213,6 +213,8 @@ int proj_update(Proj& P, const sem_coef* c, bool pairs, const double* x, const d
   double* v = P.X + (int64_t)P.count * P.nL;
   double* w = P.AX + (int64_t)P.count * P.nL;
   SEM_CUDA_TRY(cudaMemcpyAsync(v, src, P.nL * 8, cudaMemcpyDeviceToDevice, s));
+  // the even-odd operator whatever the solve's: a space serves solves of any tolerance, those above 1e-9 keep their result bit for
+  // bit (solve.cu), and A v differs between the operators by FP64 roundings only
   if (pairs) SEM_TRY(ax_pairs_apply(L, v, w, c->h1, c->h2, c->h1_L, s, true));
   else SEM_TRY(ax_apply(L, SEM_FP64, v, w, c->h1, c->h2, c->h1_L, s, nullptr, true));
   SEM_TRY(gs_apply(L, SEM_FP64, w, true, s));

@@ -345,7 +345,9 @@ int precond_setup(Ctx& C, double h1, double h2, int prec, cudaStream_t s, const 
   // level operators take it point by point (the scalar h1 becomes 1)
   C.pc_nodal = h1L != nullptr;
   C.pc_h1L = h1L;
-  const bool eo = !h1L && prec != SEM_FP64;   // the eigenvalue bounds of an FP32 V-cycle keep their last bit (see solve_impl)
+  // the eigenvalue bounds of an FP32 V-cycle keep their last bit: the set-up does not know the tolerance, and a solve above 1e-9
+  // keeps its result (see solve_impl)
+  const bool eo = !h1L && prec != SEM_FP64;
   if (h1L) {
     h1 = 1.0;
     for (int l = 0; l < C.nlevels; ++l) {
@@ -749,10 +751,11 @@ int solve_impl(Ctx* C, Proj* P, const double* f, const sem_coef* c, double tol, 
     return SEM_EINVAL;
   }
   // Outer operator R QQ^T A_L p. An FP32 V-cycle turns a last-bit change of its input into other FP32 roundings and another
-  // number of coarse iterations, and the solution then changes by a part of the solve's own error (3e-8 to 9e-8 at
-  // tol = 1e-8, 24^3, whichever two FP64-accurate operators are compared). So such a solve to a loose tolerance keeps the
-  // even-odd operator and its earlier result; below 1e-9 (5e-12 apart at 1e-10), with an FP64 V-cycle and with Jacobi the digit
-  // operator runs.
+  // number of coarse iterations, and the solution then moves by a part of the solve's own error, whichever two FP64-accurate
+  // operators are compared: 3e-8 to 9e-8 at tol = 1e-8 (24^3). Above 1e-9 such a solve keeps the even-odd (or pair) operator, so
+  // that its result stays what it was, bit for bit; this is a choice of reproducibility, not of accuracy, and costs what the header
+  // says. Tighter ones, where an operator application is a larger part and the move is below 1e-8 (64 solves of four meshes: up
+  // to 8e-9 at 1e-9, 4e-9 at 5e-10, 1.7e-9 at 1e-10, median 1e-13), those with an FP64 V-cycle and Jacobi take the digits.
   const bool eo = precond == SEM_PC_PMG && prec != SEM_FP64 && tol > 1e-9;
   auto outer_ax = [&](const double* in, double* out, const double* skip, cudaStream_t st) -> int {
     if (pairs) SEM_TRY(ax_pairs_apply(C->lev[0], in, out, c->h1, c->h2, c->h1_L, st, eo));
