@@ -52,8 +52,8 @@ __device__ __forceinline__ bool dig_h1_wide(const uint32_t high, const uint32_t 
 // exponent of a scalar h1, as the kernel takes it (4096: not a normal number, the elements go to the FP64 form)
 inline int dig_h1_exp(double h1) { return h1 == 0.0 ? 0 : std::isnormal(h1) ? std::ilogb(h1) : 4096; }
 
-// Elements the fixed-point form does not take. nil: no high word of u is set (and all else is within fixed point): the element is
-// zero, unless some value is below 2^-1042.
+// Elements the fixed-point form does not take. nil: no high word of u is set and h1 and G are finite: the element is zero, unless some
+// value is below 2^-1042.
 template <int NP, bool VARH1>
 __device__ __noinline__ void dig_fallback(double* A, int e, const double* u, double* w, const double* G,
                                           const EOMat<ArF64>& Df, const EOMat<ArF64>& Dt, double h1, double h2,
@@ -176,16 +176,16 @@ __device__ __forceinline__ bool dig_element(const int e, const double* __restric
     }
   }
   // biased exponent of the largest |u|, one more where its fixed-point form would reach 2^63 (1 - 2^-7)
-  const int eu = um ? (int)((um + 0x4000) >> 20) : 1023;
+  const int eu = (int)((um + 0x4000) >> 20);   // no high word set: 0, not held
   const int eh = VARH1 ? (hm ? (int)(hm >> 20) - 1022 : 0) : 0;   // |h1| < 2^eh
   // exponent of the result's unit before the shift by the derivatives' size (at most 32)
   const int ex = ge + eh + eu - 1023 - kexp - DIG_SH2 - 12;
-  const bool off = hm >= 0x7ff00000u || ge == DIG_BAD || abs(ex) > 800 || abs(ex + e1) > 800 || abs(eh) > 800 ||
-                   abs(eu - 1023) > 800 || (VARH1 && dig_h1_wide(hm, hl, span));
-  if (um - 1u >= 0x7fefffffu || off) {   // um zero, or that of an Inf or NaN
+  if (um >= 0x7ff00000u || hm >= 0x7ff00000u || ge == DIG_BAD || abs(ex) > 800 || abs(ex + e1) > 800 ||
+      abs(eh) > 800 || abs(eu - 1023) > 800 || (VARH1 && dig_h1_wide(hm, hl, span))) {
+    const bool nil = um == 0 && hm < 0x7ff00000u && ge != DIG_BAD && e1 < 4096;
     const ptrdiff_t at = (ptrdiff_t)e * NP3 + loc;
     dig_fallback<NP, VARH1>(reinterpret_cast<double*>(smem), e, u - at, w - at, G, Df, Dt, h1, h2,
-                            VARH1 ? h1L - at : nullptr, !off && um == 0);
+                            VARH1 ? h1L - at : nullptr, nil);
     return false;
   }
 

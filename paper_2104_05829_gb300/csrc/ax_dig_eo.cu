@@ -3,7 +3,7 @@
 // What bounds it: the FP64 form (ax_eo.cu) issues an FP64 instruction every 16 cycles: 2,368 us at 26^3, N = 9, against 187 us
 // for its bytes. Here it is instruction issue and the mma.sync chains (ncu, 16^3, N = 9: issue 56 %, tensor pipe 30 %, 755 warp
 // instructions for 32 points; 917 with one loop over all groups and 8-byte stores). Element kernel, about 16 million points, FP64 form ->
-// this: N = 8 1841 -> 675 us, N = 9 2368 -> 602, N = 10 1872 -> 653, N = 11 2460 -> 491. (The FP32-pair kernel: 458, 634, 495, 682.)
+// this: N = 8 1841 -> 675 us, N = 9 2368 -> 603, N = 10 1872 -> 654, N = 11 2460 -> 491. (The FP32-pair kernel: 458, 634, 495, 682.)
 // Error against 128-bit arithmetic, 2-norm, 4x3x4 warped elements: random u 0.57e-16 to 0.7e-16 (FP64 form 1.4e-16 to 1.65e-16); linear,
 // quadratic and smooth u 0.54e-15 (N = 8) to 5.3e-15 (N = 11) (FP64 form 2.9e-15 to 1.8e-14).
 //
@@ -47,8 +47,9 @@ struct DigEoShape {
   static constexpr size_t SMEM = 8 * (size_t)(4 * FLD > EO ? 4 * FLD : EO);
 };
 
-// Blocks an SM, as many as the fields let in: the warps wait on mma.sync chains (N = 9, 26^3: 648, 617, 600 us at four, five, six;
-// N = 11, 21^3: 535 at two, 490 at three; N = 10, 23^3: 775 at three, 652 at four).
+// Blocks an SM, as many as the fields let in: the warps wait on mma.sync chains (each before the room for mirror sums, which costs
+// two microseconds at any: N = 9, 26^3: 648, 617, 600 us at four, five, six; N = 11, 21^3: 535 at two, 490 at three; N = 10, 23^3: 775 at
+// three, 652 at four).
 template <int NP>
 constexpr int dig_eo_min_blocks() {
   return NP == 12 ? 3 : NP == 11 ? 4 : 6;
@@ -207,13 +208,13 @@ __global__ void __launch_bounds__(DigEoShape<NP>::T, dig_eo_min_blocks<NP>())
       hl = max(hl, s_max[3][t]);
     }
   }
-  const int eu = um ? (int)((um + 0x4000) >> 20) : 1023;
+  const int eu = (int)((um + 0x4000) >> 20);
   const int eh = VARH1 ? (hm ? (int)(hm >> 20) - 1022 : 0) : 0;   // |h1| < 2^eh
   const int ex = ge + eh + eu - 1023 - kexp - DIG_SH2 - 12 + 2;   // values and fluxes carry half
-  const bool off = hm >= 0x7ff00000u || ge == DIG_BAD || abs(ex) > 800 || abs(ex + e1) > 800 || abs(eh) > 800 ||
-                   abs(eu - 1023) > 800 || (VARH1 && dig_h1_wide(hm, hl, span));
-  if (um - 1u >= 0x7fefffffu || off) {   // um zero, or that of an Inf or NaN
-    dig_fallback<NP, VARH1>(reinterpret_cast<double*>(dig_eo_smem), e, u, w, G, Df, Dt, h1, h2, h1L, !off && um == 0);
+  if (um >= 0x7ff00000u || hm >= 0x7ff00000u || ge == DIG_BAD || abs(ex) > 800 || abs(ex + e1) > 800 ||
+      abs(eh) > 800 || abs(eu - 1023) > 800 || (VARH1 && dig_h1_wide(hm, hl, span))) {
+    const bool nil = um == 0 && hm < 0x7ff00000u && ge != DIG_BAD && e1 < 4096;
+    dig_fallback<NP, VARH1>(reinterpret_cast<double*>(dig_eo_smem), e, u, w, G, Df, Dt, h1, h2, h1L, nil);
     return;
   }
 #pragma unroll
