@@ -4,8 +4,8 @@
 // What bounds it: the FP64 form (ax_eo.cu) issues about 50 FP64 instructions a point at 16 cycles a warp and SM each, eight
 // times the time of its bytes. Here 32 points cost 30 mma.sync (2.3 cycles each), 27 IMAD.WIDE (1.3, and not beside an
 // mma.sync), about 280 other 32-bit instructions and four FP64 ones (16): 184 cycles at 24 warps an SM, of which
-// the tensor and wide-multiply pipes need 110 and the bytes 107. Element kernel at 32^3, N = 7: 1576 -> 306 us (2.8 TB/s); 43^3,
-// N = 5: 1444 -> 617 us (padded to 64 lines of 8 points); the FP32-pair kernel takes 366 and 350 us there.
+// the tensor and wide-multiply pipes need 110 and the bytes 107. Element kernel at 32^3, N = 7: 1576 -> 309 us (3.9 TB/s); 43^3,
+// N = 5: 1444 -> 608 us (padded to 64 lines of 8 points); the FP32-pair kernel takes 366 and 353 us there.
 //
 // One element per block, one warp per two planes k = 2w, 2w+1; lane (g, c) holds the points
 // (i, j) = (2c, g), (2c+1, g) of both planes all the way, the layout of an mma's rows and results:
@@ -21,8 +21,8 @@
 // The GLL weights make G, and the result, a hundred times smaller at an element's edges and corners than inside. So G is stored
 // over 2^(a_i + a_j + a_k), 2^a_i near rho_i^(3/4) (a power of two: no rounding), the second contraction uses
 // 2^-a D^T 2^a, and the result gets 2^(a_i + a_j + a_k) back in the exponent of its scale: edges and corners then keep the
-// relative error of the interior (2-norm error against 80-bit arithmetic on random u: 0.7e-16 of the result, 1.6e-16 for
-// the FP64 form; smooth u 2e-16 and 6e-15).
+// relative error of the interior (2-norm error against 128-bit arithmetic, N = 4 and 7: random u 0.5e-16 and 0.6e-16 of the result,
+// 1.3e-16 and 1.4e-16 for the FP64 form; linear, quadratic and smooth u 0.6e-16 to 2.6e-16, FP64 form 0.9e-15 to 8.5e-15).
 //
 // Elements that fixed point cannot hold (an Inf or NaN in u, h1 or G, exponents near the ends of the FP64 range, or a nodal h1
 // that spans more than 2^8) are computed by the even-odd FP64 code in the same block. The look at h1's span costs a nodal call 0.4 to
@@ -43,7 +43,7 @@ int ax_dig_eo_apply(const Level& L, int e0, int E, const double* u, double* w, d
 namespace {
 
 // Blocks an SM. The warps wait on mma.sync chains and on each other, so more of them pay for a few spilled registers
-// (N = 7, 32^3: 327 us at five blocks, 306 at six (80 registers), 316 at seven; N = 5, 43^3: 648, 643, 617, 615 at 5..8).
+// (N = 7, 32^3, with the kernel at 306 us: 327 us at five blocks, 306 at six (80 registers), 316 at seven; N = 5, 43^3: 648, 643, 617, 615 at 5..8).
 template <int NP>
 constexpr int dig_min_blocks() {
   return NP <= 6 ? 7 : 6;
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(128)
 struct DigHost {
   int dg[2][12][12][8];   // digits of the scaled matrices [stage][out][in]
   int kexp;               // c1 c2 = 2^kexp
-  int a[12];              // 2^a next to the GLL weights
+  int a[12];              // 2^a next to the GLL weights^(3/4)
 };
 
 // D scaled by c1 = 2^k / c2 and 2^-a D^T 2^a by c2: every entry below 1 (eight digits), a line's derivative below 2 max|u|

@@ -1,7 +1,7 @@
 // FP64 element operator in integer digits (dig.cuh, ax_dig.cu) for 8 <= N <= 11, with even-odd lines.
 //
 // What bounds it: the FP64 form (ax_eo.cu) issues an FP64 instruction every 16 cycles: 2,368 us at 26^3, N = 9, against 187 us
-// for its bytes. Here it is instruction issue and the mma.sync chains (ncu, 16^3, N = 9: issue 56 %, tensor pipe 30 %, 755 warp
+// for its bytes. Here it is instruction issue and the mma.sync chains (ncu, 16^3, N = 9: issue 56 %, tensor pipe 30 %, 758 warp
 // instructions for 32 points; 917 with one loop over all groups and 8-byte stores). Element kernel, about 16 million points, FP64 form ->
 // this: N = 8 1841 -> 675 us, N = 9 2368 -> 603, N = 10 1872 -> 654, N = 11 2460 -> 491. (The FP32-pair kernel: 458, 634, 495, 682.)
 // Error against 128-bit arithmetic, 2-norm, 4x3x4 warped elements: random u 0.57e-16 to 0.7e-16 (FP64 form 1.4e-16 to 1.65e-16); linear,

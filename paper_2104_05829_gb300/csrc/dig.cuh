@@ -31,7 +31,7 @@ namespace sem {
 constexpr int DIG_SH1 = 46, DIG_SH2 = 47;   // scale 2^SH of the leading digit products in a merged sum, per stage
 
 // One order's matrices in digits: stage 0 multiplies by D (scaled by c1), stage 1 by 2^-a D^T 2^a (scaled by
-// c2), c1 c2 = 2^k; 2^a_i is the power of two next to the GLL weight rho_i (see ax_dig.cu).
+// c2), c1 c2 = 2^k; 2^a_i is the power of two next to (rho_i / max rho)^(3/4), rho the GLL weights (see ax_dig.cu).
 struct DigTab {
   uint4 frag[2][4][32];          // [stage][m][lane (g, c)]: (odd, even) rows of output g for input points 2c, 2c+1
   unsigned long long nk0[8];     // stage 0: minus the merged sum of an all-zero line, per output

@@ -11,8 +11,8 @@
 // Every block adds all the parts in the same fixed order, so all take the same alpha and beta and leave in the same
 // iteration. A wait is bounded (sem_opts.spin_limit). x, r and the scalars are written only once all blocks are through (jac_commit); when
 // a wait gives up, all blocks leave without a write to them, and the kernels without waits take the solve over from there.
-// Measured, an iteration: N = 7, one element 32.8 -> 11.0 us, 4^3 36.9 -> 14.4, 6^3 42.5 -> 17.9, 8^3 55.0 -> 25.3 (the manufactured
-// 4^3 solve 6.9 -> 2.8 ms). What is left at one element is latency: the operator's chain, two barriers and four
+// Measured, an iteration: N = 7, one element 32.8 -> 11 to 12 us, 4^3 36.9 -> 14.7, 6^3 42.5 -> 18.2, 8^3 55.0 -> 25.4 (the manufactured
+// 4^3 solve 6.9 -> 2.73 ms). What is left at one element is latency: the operator's chain, two barriers and four
 // reductions; at four elements an SM the FP64 instructions of the vector work (about 400 a block, 16 cycles each), so sums
 // are formed by one warp where one is enough and the quotients by one lane.
 #include "ax_dig.cuh"
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(DigShape<NP>::T, JAC_MIN_BLOCKS)
 // waits gave up leaves x, r and the scalars as they were (S_ITER and S_DONE tell) and p undefined: jacobi_dig_resume makes it D^-1 r.
 //
 // The rule. All blocks must be resident, four on an SM: up to 608 elements on 152 SMs. It is the faster form over that whole
-// range (N = 7, 8 x 8 x 9 elements: 27.2 against 57.2 us an iteration; N = 4, 5, 6, 8^3: 21.9, 22.4, 25.0 against 43.0, 44.1, 49.1).
+// range (N = 7, 8 x 8 x 9 elements: 27.1 against 57.2 us an iteration; N = 4, 5, 6, 8^3: 21.2, 22.4, 24.6 against 43.0, 44.1, 49.1).
 // A spin limit under a millisecond could run out in an ordinary solve: it keeps the launches, which have no waits. A limit of
 // zero does not: every barrier gives up at the first poll that finds a block missing, and the launches take over.
 int jacobi_dig_solve(Ctx& C, const Level& L, double* x, double* r, double* p, double* w, const double* dinv, double h1,

@@ -14,8 +14,8 @@
 
 namespace sem {
 
-struct DigTab;
-struct DigEoTab;      // dig.cuh
+struct DigTab;      // dig.cuh
+struct DigEoTab;    // ax_dig_eo.cu
 struct AdvDigTab;   // advect_dig.cu
 
 // ----------------------------------------------------------------------------
@@ -262,10 +262,10 @@ int ax_eo_apply_range(const Level& L, int e0, int e1, const double* u, double* w
 // ---- ax_dig.cu (FP64 element operator in integer digits on the tensor cores)
 int dig_build(Level& L, cudaStream_t s);
 // N = 7 and 11, and N = 9 from 2,048 elements: the digit kernels answer the FP32-pair calls too, with more bits and in less time
-// (306 against 366 us at 32^3, 600 against 635 at 26^3, 490 against 682 at 21^3). At N = 9 a block's chain of line groups is the
+// (309 against 366 us at 32^3, 603 against 635 at 26^3, 491 against 682 at 21^3). At N = 9 a block's chain of line groups is the
 // longer one, which shows while the device is not full (36 elements 16.4 against 13.4 us, 1,210 51.5 against 50.1, 2,184 89.6
 // against 93.9; N = 7: 9.9 against 12.3 at 36, N = 11: 18.5 against 18.5). At other orders the lines are padded and the
-// pair kernel is the faster one (N = 5, 43^3: 617 against 350 us; N = 8, 28^3: 673 against 458; N = 10, 23^3: 652 against 495).
+// pair kernel is the faster one (N = 5, 43^3: 608 against 353 us; N = 8, 28^3: 675 against 458; N = 10, 23^3: 654 against 495).
 inline bool dig_for_pairs(const Level& L) {
   return L.Gx && (L.NP == 8 || L.NP == 12 || (L.NP == 10 && L.E >= 2048));
 }

@@ -522,7 +522,8 @@ int sem_setup(const sem_mesh* m, const sem_opts* opts_in, sem_ctx** out) {
   CUSTEP(cudaStreamCreateWithFlags(&C->cap_stream, cudaStreamNonBlocking));
   // The fixed-point factors come after everything else: allocated between the other arrays (right behind G) they left the FP32-pair
   // advection of an N = 8 box of 384 elements at 2,840 us a substep against 2,520 without them, and 2,371 from here; an
-  // 18 x 11 x 16 p-MG solve of order 5 took 7.50 ms either way and takes 7.21. Same kernels, same bits: where the arrays lie.
+  // 18 x 11 x 16 p-MG solve of order 5 took 7.50 ms either way and takes 7.21. Same kernels, same bits; what about an array's place
+  // makes the difference was not found, so the order promises nothing to the next array.
   for (int l = 0; l < C->nlevels; ++l) STEP(dig_build(C->lev[l], s));
   CUSTEP(cudaStreamSynchronize(s));
   cudaStreamDestroy(s);
